@@ -6,11 +6,11 @@
 // CTA, so the result does not depend on scheduling.
 //
 // S(k) = |sum_r (phi - mean) e^{-i k.r}|^2 / N: the FFT runs in FP64 on the
-// GPU, line by line along each axis, each line transformed in shared memory
-// by a mixed-radix Cooley-Tukey (decimation in time, digit-reversed load).
+// GPU on the half spectrum of the real field (lf_fft.cu).
 // The k = 0 coefficient, the only one the mean affects, is left out of the
 // shells.  Shells have width dk = 2 pi / L_min; bin b = floor(|k|/dk + 1/2),
 // b = 1 .. L_min/2.
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "lf_diag.cuh"
+#include "lf_fft.cuh"
 
 namespace lf {
 
@@ -25,16 +26,14 @@ namespace {
 
 constexpr int kBlocks = 152 * 8;   // partial sums: a few waves on 152 SMs
 constexpr int kThreads = 256;
-constexpr int kMaxRadix = 32;
-constexpr int kMaxStages = 40;
-constexpr int kShellSmemBins = 4096;   // shell histogram kept in shared memory up to this many bins
+constexpr int kMaxBins = 2048;     // of S(k): half the longest line the FFT takes
 
 struct Scratch {
     double* part;    // kBlocks * DQ_N
     double* res;     // DQ_N
     double* layers;  // L * 2
     double* bins;    // (B + 1) * 2: sum, count
-    double2* fft;    // N
+    double2* fft;    // half spectrum (nx / 2 + 1) ny nz <= N
 };
 
 size_t a256(size_t v) { return (v + 255) / 256 * 256; }
@@ -193,166 +192,64 @@ __global__ void __launch_bounds__(kThreads) k_layers(Geom g, const R* __restrict
     block_reduce_store<2>(v, out + 2 * h, -1);
 }
 
-// ---- FFT ------------------------------------------------------------------
-struct FftPlan {
-    int n;
-    int nst;
-    int radix[kMaxStages];
-};
-
-bool make_plan(int n, FftPlan* p)
+// ---- structure factor --------------------------------------------------------
+__device__ __forceinline__ double kfreq2(int i, int n, int64_t lmin)
 {
-    p->n = n;
-    p->nst = 0;
-    int m = n;
-    while (m % 4 == 0) { p->radix[p->nst++] = 4; m /= 4; }
-    for (int r = 2; r <= kMaxRadix && m > 1; ++r)
-        while (m % r == 0) {
-            if (p->nst >= kMaxStages) return false;
-            p->radix[p->nst++] = r;
-            m /= r;
-        }
-    return m == 1;
-}
-
-__device__ __forceinline__ double2 cmul(double2 a, double2 b)
-{
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-// multiply by -i
-__device__ __forceinline__ double2 cmul_mi(double2 a) { return make_double2(a.y, -a.x); }
-
-// C lines of length n per CTA; line l starts at (l / inner) * outer_stride +
-// (l % inner) * inner_stride and has element stride `es`.  Shared memory:
-// the twiddle table tw[j] = e^{-2 pi i j / n}, j < n, then the C lines.
-__global__ void k_fft_lines(double2* data, FftPlan plan, int64_t es, int64_t nlines, int64_t inner,
-                            int64_t inner_stride, int64_t outer_stride, int C)
-{
-    extern __shared__ double2 smem_fft[];
-    const int n = plan.n;
-    double2* tw = smem_fft;
-    double2* buf = smem_fft + n;
-    const int64_t l0 = (int64_t)blockIdx.x * C;
-    const int nl = (int)((nlines - l0) < C ? (nlines - l0) : C);
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double sn, cs;
-        sincospi(-2.0 * (double)j / (double)n, &sn, &cs);
-        tw[j] = make_double2(cs, sn);
-    }
-    // digit-reversed load
-    for (int t = threadIdx.x; t < nl * n; t += blockDim.x) {
-        int c, j;
-        if (es == 1) { c = t / n; j = t - c * n; }
-        else { j = t / nl; c = t - j * nl; }
-        const int64_t l = l0 + c;
-        const int64_t base = (l / inner) * outer_stride + (l % inner) * inner_stride;
-        int pos = 0, rem = j, size = n;
-        for (int st = plan.nst - 1; st >= 0; --st) {
-            const int r = plan.radix[st];
-            size /= r;
-            pos += (rem % r) * size;
-            rem /= r;
-        }
-        buf[c * n + pos] = data[base + (int64_t)j * es];
-    }
-    __syncthreads();
-    int m = 1;
-    for (int st = 0; st < plan.nst; ++st) {
-        const int r = plan.radix[st];
-        const int nb = n / r;
-        const int stride = n / (m * r);          // tw index step of W_{m r}
-        for (int t = threadIdx.x; t < nl * nb; t += blockDim.x) {
-            const int c = t / nb, bi = t - c * nb;
-            const int grp = bi / m, k = bi - grp * m;
-            double2* b = buf + c * n + grp * m * r + k;
-            if (r == 2) {
-                const double2 y0 = b[0], y1 = cmul(b[m], tw[k * stride]);
-                b[0] = cadd(y0, y1);
-                b[m] = csub(y0, y1);
-            } else if (r == 4) {
-                const double2 y0 = b[0];
-                const double2 y1 = cmul(b[m], tw[k * stride]);
-                const double2 y2 = cmul(b[2 * m], tw[2 * k * stride]);
-                const double2 y3 = cmul(b[3 * m], tw[3 * k * stride]);
-                const double2 a0 = cadd(y0, y2), a1 = csub(y0, y2);
-                const double2 b0 = cadd(y1, y3), b1 = cmul_mi(csub(y1, y3));
-                b[0] = cadd(a0, b0);
-                b[m] = cadd(a1, b1);
-                b[2 * m] = csub(a0, b0);
-                b[3 * m] = csub(a1, b1);
-            } else {
-                double2 y[kMaxRadix];
-                y[0] = b[0];
-                for (int s2 = 1; s2 < r; ++s2) y[s2] = cmul(b[s2 * m], tw[k * s2 * stride]);
-                const int wr = n / r;            // tw index step of W_r
-                for (int q = 0; q < r; ++q) {
-                    double2 acc = y[0];
-                    for (int s2 = 1; s2 < r; ++s2) acc = cadd(acc, cmul(y[s2], tw[((q * s2) % r) * wr]));
-                    b[q * m] = acc;
-                }
-            }
-        }
-        __syncthreads();
-        m *= r;
-    }
-    for (int t = threadIdx.x; t < nl * n; t += blockDim.x) {
-        int c, j;
-        if (es == 1) { c = t / n; j = t - c * n; }
-        else { j = t / nl; c = t - j * nl; }
-        const int64_t l = l0 + c;
-        const int64_t base = (l / inner) * outer_stride + (l % inner) * inner_stride;
-        data[base + (int64_t)j * es] = buf[c * n + j];
-    }
-}
-
-template <typename R>
-__global__ void k_fft_fill(Geom g, const R* __restrict__ phi, double2* out)
-{
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = k / g.nx;
-        const int x = (int)(k - row * g.nx);
-        out[k] = make_double2((double)phi[row * g.pitch + x], 0.0);
-    }
-}
-
-__device__ __forceinline__ double kfreq2(int64_t i, int64_t n, int64_t lmin)
-{
-    const int64_t f = (2 * i <= n) ? i : i - n;
+    const int f = (2 * i <= n) ? i : i - n;
     const double r = (double)f * (double)lmin / (double)n;   // |k| / dk along this axis
     return r * r;
 }
 
-__global__ void k_shells(Geom g, const double2* __restrict__ X, int64_t lmin, int64_t B, double* bins)
+// Shell sums of |X|^2 over the half spectrum X (2 x the transform, rows of H =
+// nx / 2 + 1): a mode with a conjugate partner counts twice.  A warp takes a
+// row at a time, so its (ky, kz) part is formed once per row, the kx parts come
+// from a table, and the shell b = floor(sqrt(r2) + 1/2) from an FP32 root
+// corrected against (b - 1/2)^2 <= r2 < (b + 1/2)^2 in FP64: about ten FP64
+// operations per mode (the divisions and the FP64 root made it sixty): 114 ->
+// 32 us at 1024^2.
+__global__ void __launch_bounds__(kThreads) k_shells(Geom g, const double2* __restrict__ X, int64_t lmin, int B,
+                                                     double* __restrict__ bins)
 {
-    extern __shared__ double hist[];            // 2 (B + 1) doubles when B <= kShellSmemBins
-    const bool local = B <= kShellSmemBins;
-    if (local) {
-        for (int i = threadIdx.x; i < 2 * (B + 1); i += blockDim.x) hist[i] = 0.0;
-        __syncthreads();
+    extern __shared__ double sm[];
+    const int H = half_nx(g.nx);
+    double* sum = sm;                            // B + 1
+    double* kx2 = sum + B + 1;                   // H
+    unsigned* cnt = reinterpret_cast<unsigned*>(kx2 + H);   // B + 1
+    for (int i = threadIdx.x; i <= B; i += kThreads) { sum[i] = 0.0; cnt[i] = 0u; }
+    for (int i = threadIdx.x; i < H; i += kThreads) kx2[i] = kfreq2(i, g.nx, lmin);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int rows = g.ny * g.nz, step = gridDim.x * (kThreads / 32);
+    const double top = ((double)B + 0.5) * ((double)B + 0.5);
+    for (int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows; row += step) {
+        const int iz = row / g.ny, iy = row - iz * g.ny;
+        double rr = kfreq2(iy, g.ny, lmin);
+        if (g.d == 3) rr += kfreq2(iz, g.nz, lmin);
+        if (rr >= top) continue;
+        const double2* x = X + (int64_t)row * H;
+        for (int ix = lane; ix < H; ix += 32) {
+            const double r2 = kx2[ix] + rr;
+            if (r2 >= top) break;
+            int b = (int)(sqrtf((float)r2) + 0.5f);
+            const double e = r2 - 0.25;          // b (b - 1) <= e < b (b + 1)
+            if (e < (double)(b * (b - 1))) --b;
+            else if (e >= (double)(b * (b + 1))) ++b;
+            if (b < 1) continue;
+            const double2 v = x[ix];
+            const bool two = ix > 0 && 2 * ix < g.nx;
+            double p = v.x * v.x + v.y * v.y;
+            if (two) p += p;
+            atomicAdd(&sum[b], p);
+            atomicAdd(&cnt[b], two ? 2u : 1u);
+        }
     }
-    double* h = local ? hist : bins;
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        if (k == 0) continue;
-        const int64_t ix = k % g.nx, row = k / g.nx;
-        const int64_t iy = row % g.ny, iz = row / g.ny;
-        double r2 = kfreq2(ix, g.nx, lmin) + kfreq2(iy, g.ny, lmin);
-        if (g.d == 3) r2 += kfreq2(iz, g.nz, lmin);
-        const int64_t b = (int64_t)floor(sqrt(r2) + 0.5);
-        if (b < 1 || b > B) continue;
-        const double2 v = X[k];
-        atomicAdd(&h[2 * b], (v.x * v.x + v.y * v.y) / (double)N);
-        atomicAdd(&h[2 * b + 1], 1.0);
-    }
-    if (local) {
-        __syncthreads();
-        for (int i = threadIdx.x; i < 2 * (B + 1); i += blockDim.x)
-            if (hist[i] != 0.0) atomicAdd(&bins[i], hist[i]);
-    }
+    __syncthreads();
+    const double inv = 0.25 / ((double)g.nx * g.ny * g.nz);
+    for (int i = threadIdx.x; i <= B; i += kThreads)
+        if (cnt[i]) {
+            atomicAdd(&bins[2 * i], sum[i] * inv);
+            atomicAdd(&bins[2 * i + 1], (double)cnt[i]);
+        }
 }
 
 unsigned grid_n(int64_t N)
@@ -369,56 +266,29 @@ int64_t lmin_of(const Geom& g)
     return l;
 }
 
-// Forward DFT (kernel e^{-2 pi i j k / n}) of every line along axis a of a
-// packed [nz][ny][nx] complex FP64 array, in place.
-cudaError_t fft_lines_axis(const Geom& g, double2* data, int a, const FftPlan& plan, cudaStream_t s)
-{
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    const int n = plan.n;
-    int C = 4096 / n;
-    if (C < 1) C = 1;
-    if (C > 16) C = 16;
-    int64_t nlines, inner, inner_stride, outer_stride, es;
-    if (a == 0) { nlines = N / n; inner = 1; inner_stride = 0; outer_stride = n; es = 1; }
-    else if (a == 1) { nlines = N / n; inner = g.nx; inner_stride = 1; outer_stride = (int64_t)g.nx * g.ny; es = g.nx; }
-    else { nlines = N / n; inner = (int64_t)g.nx * g.ny; inner_stride = 1; outer_stride = 0; es = (int64_t)g.nx * g.ny; }
-    const size_t smem = sizeof(double2) * (size_t)(C + 1) * n;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_fft_lines, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    const unsigned blocks = (unsigned)((nlines + C - 1) / C);
-    k_fft_lines<<<blocks, kThreads, smem, s>>>(data, plan, es, nlines, inner, inner_stride, outer_stride, C);
-    return cudaGetLastError();
-}
-
 // FFT of phi into sc.fft and the shell sums into sc.bins (device).  Returns
-// false when a lattice size has a prime factor above kMaxRadix or a line does
-// not fit in shared memory.
+// false when a lattice size has a prime factor above 31 or a line does not
+// fit in shared memory.
 bool enqueue_sk(const DiagInput& in, const Scratch& sc, cudaStream_t s, cudaError_t* err)
 {
     const Geom& g = in.g;
     const int64_t lmin = lmin_of(g), B = lmin / 2;
     const int sizes[3] = {g.nx, g.ny, g.nz};
-    FftPlan plans[3];
-    for (int a = 0; a < g.d; ++a) {
-        if (!make_plan(sizes[a], &plans[a]) || sizes[a] > 4096) return false;   // line + twiddles fit in smem
-    }
-    *err = cudaSuccess;
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    if (in.prec == LF_FP64) k_fft_fill<double><<<grid_n(N), kThreads, 0, s>>>(g, (const double*)in.phi, sc.fft);
-    else k_fft_fill<float><<<grid_n(N), kThreads, 0, s>>>(g, (const float*)in.phi, sc.fft);
-    for (int a = 0; a < g.d; ++a) {
-        const cudaError_t e = fft_lines_axis(g, sc.fft, a, plans[a], s);
-        if (e != cudaSuccess) { *err = e; return true; }
-    }
+    for (int a = 0; a < g.d; ++a)
+        if (!fft_supported(sizes[a])) return false;
+    static_assert(kMaxBins * 2 == 4096, "B <= kMaxBins for every supported line");
+    *err = in.prec == LF_FP64 ? rfft_x<double>(g, (const double*)in.phi, sc.fft, s)
+                              : rfft_x<float>(g, (const float*)in.phi, sc.fft, s);
+    for (int a = 1; a < g.d && *err == cudaSuccess; ++a) *err = fft_axis(g, sc.fft, a, s);
+    if (*err != cudaSuccess) return true;
     cudaMemsetAsync(sc.bins, 0, sizeof(double) * 2 * (B + 1), s);
-    const size_t hs = B <= kShellSmemBins ? sizeof(double) * 2 * (B + 1) : 0;
-    if (hs > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_shells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hs);
-        if (e != cudaSuccess) { *err = e; return true; }
-    }
-    k_shells<<<grid_n(N), kThreads, hs, s>>>(g, sc.fft, lmin, B, sc.bins);
+    const size_t hs = (sizeof(double) + sizeof(unsigned)) * (B + 1) + sizeof(double) * half_nx(g.nx);
+    static unsigned long long attr_done = 0;
+    const int most = (int)((sizeof(double) + sizeof(unsigned)) * (kMaxBins + 1) + sizeof(double) * (kMaxBins + 1));
+    if ((*err = raise_smem_limit(k_shells, most, &attr_done)) != cudaSuccess) return true;
+    const int64_t warps = (int64_t)g.ny * g.nz;
+    const unsigned nblk = (unsigned)std::min<int64_t>(152 * 4, (warps + kThreads / 32 - 1) / (kThreads / 32));
+    k_shells<<<nblk, kThreads, hs, s>>>(g, sc.fft, lmin, (int)B, sc.bins);
     *err = cudaGetLastError();
     return true;
 }
@@ -452,16 +322,6 @@ size_t diag_scratch_bytes(int d, int64_t nx, int64_t ny, int64_t nz)
 }
 
 double2* fft_buffer(const Geom& g, void* scratch) { return carve(g, scratch).fft; }
-
-bool fft_supported(int n) { FftPlan p; return n <= 4096 && make_plan(n, &p); }
-
-cudaError_t fft_forward_axis(const Geom& g, double2* data, int axis, cudaStream_t s)
-{
-    const int sizes[3] = {g.nx, g.ny, g.nz};
-    FftPlan plan;
-    if (!make_plan(sizes[axis], &plan) || sizes[axis] > 4096) return cudaErrorInvalidValue;
-    return fft_lines_axis(g, data, axis, plan, s);
-}
 
 int run_diag(const DiagInput& in, DiagResult* r, cudaStream_t s)
 {

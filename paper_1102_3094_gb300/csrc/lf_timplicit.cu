@@ -8,10 +8,13 @@
 // with the same Laplacian L (compact 5-/7-point or isotropic 9-/19-point) and
 // wall rules as the explicit update.  L is diagonal in a lattice Fourier basis
 // along the periodic axes and couples only neighbouring layers along the wall
-// normal, so the solve is: FP64 DFT along x (2D) or x and y (3D); for every
-// Fourier mode a tridiagonal system along the wall normal (Thomas algorithm,
-// one thread per mode) -- or a plain division when every axis is periodic;
-// the inverse DFT as conj(DFT(conj(.))) / n; back to the state's precision.
+// normal, so the solve is: FP64 DFT along x (2D) or x and y (3D) onto the half
+// spectrum of the real field (lf_fft.cu); for every mode of it a tridiagonal
+// system along the wall normal (Thomas algorithm, one thread per mode) -- or a
+// plain division when every axis is periodic; the inverse DFT as
+// conj(DFT(conj(.))) / n; back to the state's precision.  The half spectrum
+// halves the transforms and the modes, all of which the FP64 pipe bounds:
+// 4.49 -> 1.84 ms at 256^3 with walls (transforms 3.94 -> 1.66, Thomas 0.38 -> 0.18).
 //
 // For a mode with in-plane wavenumbers (kx[, ky]) L acts on the layer
 // amplitudes as alpha (A_{j+1} + A_{j-1}) + beta A_j:
@@ -24,6 +27,7 @@
 
 #include "lf_ctx.cuh"
 #include "lf_diag.cuh"
+#include "lf_fft.cuh"
 
 namespace lf {
 
@@ -31,40 +35,20 @@ namespace {
 
 constexpr double kTwoPi = 6.283185307179586476925286766559;
 
-template <typename R>
-__global__ void k_t_load(Geom g, const R* __restrict__ T, double2* __restrict__ buf)
-{
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = k / g.nx;
-        const int x = (int)(k - row * g.nx);
-        buf[k] = make_double2((double)T[row * g.pitch + x], 0.0);
-    }
-}
-
-template <typename R>
-__global__ void k_t_store(Geom g, const double2* __restrict__ buf, double scale, R* __restrict__ T,
-                          int* __restrict__ flag)
-{
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
-    bool bad = false;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = k / g.nx;
-        const int x = (int)(k - row * g.nx);
-        const double v = buf[k].x * scale;
-        bad |= !isfinite(v);
-        T[row * g.pitch + x] = (R)v;
-    }
-    if (bad) *reinterpret_cast<volatile int*>(flag) = 1;
-}
-
 // Cosines of the wavenumbers of the mode with packed index m over the
-// periodic axes (x fastest); 1 for the others.
+// periodic axes of the half spectrum (x fastest); 1 for the others.
 __device__ __forceinline__ void mode_cos(const Geom& g, int64_t m, int nper_axes, double c[3])
 {
-    c[0] = cos(kTwoPi * (int)(m % g.nx) / g.nx);
-    c[1] = nper_axes >= 2 ? cos(kTwoPi * (int)((m / g.nx) % g.ny) / g.ny) : 1.0;
-    c[2] = nper_axes >= 3 ? cos(kTwoPi * (int)(m / ((int64_t)g.nx * g.ny)) / g.nz) : 1.0;
+    const int H = half_nx(g.nx);
+    c[0] = cos(kTwoPi * (int)(m % H) / g.nx);
+    c[1] = nper_axes >= 2 ? cos(kTwoPi * (int)((m / H) % g.ny) / g.ny) : 1.0;
+    c[2] = nper_axes >= 3 ? cos(kTwoPi * (int)(m / ((int64_t)H * g.ny)) / g.nz) : 1.0;
+}
+
+// Modes of the periodic axes when the last axis has walls.
+__host__ __device__ __forceinline__ int64_t wall_modes(const Geom& g)
+{
+    return g.d == 2 ? (int64_t)half_nx(g.nx) : (int64_t)half_nx(g.nx) * g.ny;
 }
 
 // Every axis periodic: eigenvalue of -L for mode m.
@@ -149,7 +133,7 @@ __device__ __forceinline__ double tri_diag(const TriSys& t, int j, int t_mode)
 __global__ void k_t_coef(Geom g, double* __restrict__ coef, double xi, int t_mode)
 {
     const int d = g.d;
-    const int64_t M = d == 2 ? (int64_t)g.nx : (int64_t)g.nx * g.ny;
+    const int64_t M = wall_modes(g);
     const int L = d == 2 ? g.ny : g.nz;
     const int64_t N = M * L;
     const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -174,7 +158,7 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
                            double Tw_hat0, int t_mode)
 {
     const int d = g.d;
-    const int64_t M = d == 2 ? (int64_t)g.nx : (int64_t)g.nx * g.ny;
+    const int64_t M = wall_modes(g);
     const int L = d == 2 ? g.ny : g.nz;
     const int64_t N = M * L;
     const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -258,7 +242,7 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
 // Every axis periodic: the mode is divided by 1 + xi lam; writes the conjugate.
 __global__ void k_t_divide(Geom g, double2* __restrict__ buf, double xi)
 {
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
+    const int64_t N = (int64_t)half_nx(g.nx) * g.ny * g.nz;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
         const double s = 1.0 / (1.0 + xi * lam_periodic(g, k));
         buf[k] = make_double2(buf[k].x * s, -buf[k].y * s);
@@ -287,18 +271,18 @@ int t_implicit_step(lf_ctx* c, double xi, double T_w)
 {
     const Geom& g = c->g;
     const cudaStream_t s = c->stream;
-    const int64_t N = (int64_t)g.nx * g.ny * g.nz;
     double2* buf = fft_buffer(g, c->scratch);
     R* T = (R*)c->T[c->tcur];
     const int nper_axes = g.walls ? g.d - 1 : g.d;
     int64_t nper = g.nx;
     if (nper_axes >= 2) nper *= g.ny;
     if (nper_axes >= 3) nper *= g.nz;
-    k_t_load<R><<<grid_t(N), 256, 0, s>>>(g, T, buf);
-    for (int a = 0; a < nper_axes; ++a)
-        if (fft_forward_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
+    // the transform along x is taken from T itself and gives twice the half spectrum
+    if (rfft_x<R>(g, T, buf, s) != cudaSuccess) return LF_ECUDA;
+    for (int a = 1; a < nper_axes; ++a)
+        if (fft_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
     if (g.walls) {
-        const int64_t M = N / (g.d == 2 ? g.ny : g.nz);
+        const int64_t M = wall_modes(g);
         if (!c->tcoef) return LF_EINVAL;     // lf_set_t_solver allocates the tables
         if (!c->tcoef_valid || c->tcoef_xi != xi || c->tcoef_mode != g.t_mode || c->tcoef_stencil != g.stencil) {
             k_t_coef<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, c->tcoef, xi, g.t_mode);
@@ -307,14 +291,14 @@ int t_implicit_step(lf_ctx* c, double xi, double T_w)
             c->tcoef_mode = g.t_mode;
             c->tcoef_stencil = g.stencil;
         }
-        k_t_thomas<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, buf, c->tcoef, xi, T_w * (double)nper, g.t_mode);
+        k_t_thomas<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, buf, c->tcoef, xi, 2.0 * T_w * (double)nper, g.t_mode);
     } else {
-        k_t_divide<<<grid_t(N), 256, 0, s>>>(g, buf, xi);
+        k_t_divide<<<grid_t((int64_t)half_nx(g.nx) * g.ny * g.nz), 256, 0, s>>>(g, buf, xi);
     }
-    for (int a = 0; a < nper_axes; ++a)
-        if (fft_forward_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
-    k_t_store<R><<<grid_t(N), 256, 0, s>>>(g, buf, 1.0 / (double)nper, T, c->flag_dev);
-    return cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
+    if (cudaGetLastError() != cudaSuccess) return LF_ECUDA;
+    for (int a = 1; a < nper_axes; ++a)
+        if (fft_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
+    return irfft_x<R>(g, buf, 0.5 / (double)nper, T, c->flag_dev, s) == cudaSuccess ? LF_OK : LF_ECUDA;
 }
 
 template int t_implicit_step<float>(lf_ctx*, double, double);
