@@ -71,6 +71,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ens_march2d_iso(const EnsRun* __re
                                                              const EnsItem* __restrict__ items, int nitems)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const EnsItem w = items[it];
         const EnsRun r = runs[w.run];
@@ -80,6 +81,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ens_march2d_iso(const EnsRun* __re
             march::march2d_pair_iso<NT, kD, false>(r.g, r.p, r.io, w.strip, w.pair, w.npairs, smem_raw);
         __syncthreads();   // the next item reuses the shared rings
     }
+    chain_next();
 }
 constexpr auto kIso64 = k_ens_march2d_iso<64, 6>;
 constexpr auto kIso128 = k_ens_march2d_iso<128, 3>;
@@ -89,6 +91,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ens_march2d(const EnsRun* __restri
                                                          const EnsItem* __restrict__ items, int nitems)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const EnsItem w = items[it];
         const EnsRun r = runs[w.run];
@@ -98,6 +101,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ens_march2d(const EnsRun* __restri
             march::march2d_pair<NT, kD, false>(r.g, r.p, r.io, w.strip, w.pair, w.npairs, smem_raw);
         __syncthreads();   // the next item reuses the shared rings
     }
+    chain_next();
 }
 // the single-run launcher's instantiations: 64 threads at six CTAs per SM, 128 at three
 constexpr auto kEns64 = k_ens_march2d<64, 6>;
@@ -115,6 +119,8 @@ int pairs_for(int ny, int H)
 __global__ void __launch_bounds__(256) k_ens_tsub2d(const EnsT* __restrict__ runs, const EnsTItem* __restrict__ items,
                                                    int nitems)
 {
+    chain_next();
+    chain_wait();
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const EnsTItem w = items[it];
         const EnsT r = runs[w.run];
@@ -191,22 +197,24 @@ int capture(lf_ens* e, const std::vector<int>& halves, const Half* H, const std:
     if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LF_ECUDA;
     for (int h : halves) {
         if (e->nitems[0] > 0)
-            kEns64<<<e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->stream>>>(H[h].runs, e->d_items[0], e->nitems[0]);
+            launch_chained(kEns64, e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->stream, H[h].runs, e->d_items[0],
+                           e->nitems[0]);
         if (e->nitems[1] > 0)
-            kEns128<<<e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->stream>>>(H[h].runs, e->d_items[1],
-                                                                               e->nitems[1]);
+            launch_chained(kEns128, e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->stream, H[h].runs, e->d_items[1],
+                           e->nitems[1]);
         if (e->nitems[2] > 0)
-            kIso64<<<e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->stream>>>(H[h].runs, e->d_items[2], e->nitems[2]);
+            launch_chained(kIso64, e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->stream, H[h].runs, e->d_items[2],
+                           e->nitems[2]);
         if (e->nitems[3] > 0)
-            kIso128<<<e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->stream>>>(H[h].runs, e->d_items[3],
-                                                                              e->nitems[3]);
+            launch_chained(kIso128, e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->stream, H[h].runs, e->d_items[3],
+                           e->nitems[3]);
         for (size_t s = 0; s < H[h].ts.size(); ++s) {
             if (ntitems[s] == 0) continue;
             const int blocks = std::min(ntitems[s], 152 * 8);
-            k_ens_tsub2d<<<blocks, 256, 0, e->stream>>>(H[h].ts[s], titems[s], ntitems[s]);
+            launch_chained(k_ens_tsub2d, blocks, 256, 0, e->stream, H[h].ts[s], titems[s], ntitems[s]);
         }
     }
-    cudaError_t err = cudaStreamEndCapture(e->stream, &graph);
+    cudaError_t err = cudaStreamEndCapture(e->stream, &graph);   // reports a failed launch too
     if (err != cudaSuccess) return LF_ECUDA;
     err = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);

@@ -212,4 +212,44 @@ inline cudaError_t device_sms(int* sms)
     return cudaSuccess;
 }
 
+// ---------------------------------------------------------------------------
+// Overlapped launches.  The kernels of a step are short (2 to 30 us on small
+// and middle lattices) and each depends on the one before, so the gap between
+// them counts.  A kernel launched by launch_chained may be scheduled once every
+// block of its predecessor on the stream has called chain_next() or ended; it
+// calls chain_wait() before it touches memory that another kernel writes,
+// which waits until every earlier grid has finished and its writes are
+// visible.  Everything after that is ordered as in a plain launch, also when
+// the predecessor is a kernel or copy that knows nothing of this.  (A pointer
+// to such memory is not declared __restrict__ in the kernel's parameters: the
+// compiler may load through those ahead of the wait.)
+//
+// Where chain_next() stands: at the end of the kernels whose blocks fill the
+// SMs once or twice, because blocks of the successor that come in earlier take
+// the places that happen to be free and then run unevenly spread (2D march at
+// 1024^2: 26.7 us a step with it at the end, 31.7 two rows before the end, 39
+// at the start; 28.8 without any of this); at the start of kernels with many
+// waves of small blocks or hardly any work in each.
+// 64^2 FP64 24.6 -> 21.6 us a step, 256^2 FP32 10.3 -> 8.7, 1024^2 28.8 -> 26.7,
+// 32 x 32 x 256 with eight temperature sub-steps 75 -> 57.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 }  // namespace lf

@@ -51,7 +51,9 @@ template <typename R, int TX, int TY, int NT, bool AUX, bool ISO>
 __global__ void __launch_bounds__(NT) k_step2d(Geom g, Phys<R> p, StepIO<R> io)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     tile::step2d_tile<R, TX, TY, NT, AUX, ISO>(g, p, io, blockIdx.x, blockIdx.y, smem_raw);
+    chain_next();
 }
 
 // Row-marching variant (the default for lf_step): see lf_march2d.cuh.
@@ -59,7 +61,9 @@ template <typename R, int NT, int D>
 __global__ void __launch_bounds__(NT) k_march2d(Geom g, Phys<R> p, StepIO<R> io, int H)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     march::march2d_segment<R, NT, D>(g, p, io, blockIdx.x, blockIdx.y, H, smem_raw);
+    chain_next();
 }
 
 // The row march with the isotropic 9-point stencils: see lf_march2d_iso.cuh.
@@ -67,7 +71,9 @@ template <typename R, int NT, int D>
 __global__ void __launch_bounds__(NT) k_march2d_iso(Geom g, Phys<R> p, StepIO<R> io, int H)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     march::march2d_segment_iso<R, NT, D>(g, p, io, blockIdx.x, blockIdx.y, H, smem_raw);
+    chain_next();
 }
 
 // The isotropic row march on two segments per CTA (packed FP32x2 lanes).
@@ -75,7 +81,9 @@ template <int NT, int D, bool HYDRO, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_march2d_iso_x2(Geom g, Phys<float> p, StepIO<float> io, int npairs)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     march::march2d_pair_iso<NT, D, HYDRO>(g, p, io, blockIdx.x, blockIdx.y, npairs, smem_raw);
+    chain_next();
 }
 
 // Two segments per CTA in the lanes of float2 (packed FP32x2 arithmetic).
@@ -83,7 +91,9 @@ template <int NT, int D, bool HYDRO, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_march2d_x2(Geom g, Phys<float> p, StepIO<float> io, int npairs)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    chain_wait();
     march::march2d_pair<NT, D, HYDRO>(g, p, io, blockIdx.x, blockIdx.y, npairs, smem_raw);
+    chain_next();
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
@@ -100,8 +110,7 @@ cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<fl
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    kern<<<grid, NT, M::BYTES, s>>>(g, p, io, npairs);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -116,8 +125,7 @@ cudaError_t launch_march(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    kern<<<grid, NT, M::BYTES, s>>>(g, p, io, H);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, H);
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
@@ -134,8 +142,7 @@ cudaError_t launch_march_iso_x2(const Geom& g, const Phys<float>& p, const StepI
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    kern<<<grid, NT, M::BYTES, s>>>(g, p, io, npairs);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -150,8 +157,7 @@ cudaError_t launch_march_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    kern<<<grid, NT, M::BYTES, s>>>(g, p, io, H);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, H);
 }
 
 template <typename R, int TX, int TY, int NT, bool AUX, bool ISO>
@@ -163,28 +169,31 @@ cudaError_t launch_cfg(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cud
     const cudaError_t e = raise_smem_limit(kern, (int)bytes, &attr_done);
     if (e != cudaSuccess) return e;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY);
-    kern<<<grid, NT, bytes, s>>>(g, p, io);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, bytes, s, g, p, io);
 }
 
 // ---------------------------------------------------------------------------
 // Extra temperature sub-steps (xi/nsub each) when nsub > 1.
 // ---------------------------------------------------------------------------
 template <typename R>
-__global__ void k_tsub2d(Geom g, Phys<R> p, const R* __restrict__ Tin, R* __restrict__ Tout)
+__global__ void k_tsub2d(Geom g, Phys<R> p, const R* Tin, R* Tout)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    chain_next();
+    chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     march::tsub2d_site(g, p, Tin, Tout, x, y);
 }
 
 // The same sub-step with the isotropic 9-point Laplacian (lf_tile2d.cuh).
 template <typename R>
-__global__ void k_tsub2d_iso(Geom g, Phys<R> p, const R* __restrict__ Tin, R* __restrict__ Tout)
+__global__ void k_tsub2d_iso(Geom g, Phys<R> p, const R* Tin, R* Tout)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    chain_next();
+    chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     tile::tsub2d_site_iso(g, p, Tin, Tout, x, y);
 }
@@ -238,11 +247,8 @@ cudaError_t launch_tsub(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, 
 {
     if (g.d == 3) return launch_tsub3d<R>(g, p, Tin, Tout, s);
     dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8);
-    if (g.stencil == LF_STENCIL_ISOTROPIC)
-        k_tsub2d_iso<R><<<grd, blk, 0, s>>>(g, p, Tin, Tout);
-    else
-        k_tsub2d<R><<<grd, blk, 0, s>>>(g, p, Tin, Tout);
-    return cudaGetLastError();
+    return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub2d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
+                                             : launch_chained(k_tsub2d<R>, grd, blk, 0, s, g, p, Tin, Tout);
 }
 
 template cudaError_t launch_step2d<float>(const Geom&, const Phys<float>&, const StepIO<float>&, bool, cudaStream_t);

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? (ISO ? 2 : 3) : 1)
         if (q < W4) colmap[q] = wrap_any3(x0 - 4 + q, nx);
         else rowmap[q - W4] = wrap_any3(y0 - 4 + (q - W4), ny);
     }
+    chain_wait();
     __syncthreads();
 
     // plane ring slots are counted from kbeg
@@ -475,16 +476,17 @@ cudaError_t launch_cfg3(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cu
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
-    kern<<<grid, NT, P3::BYTES, s>>>(g, p, io, Hz);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, NT, P3::BYTES, s, g, p, io, Hz);
 }
 
 template <typename R>
-__global__ void k_tsub3d(Geom g, Phys<R> p, const R* __restrict__ Tin, R* __restrict__ Tout)
+__global__ void k_tsub3d(Geom g, Phys<R> p, const R* Tin, R* Tout)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
+    chain_next();
+    chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch;
     const int zs = ny * pitch;                   // 32-bit offsets: Q * padded sites < 2^31 (checked at creation)
@@ -513,11 +515,13 @@ __global__ void k_tsub3d(Geom g, Phys<R> p, const R* __restrict__ Tin, R* __rest
 // The same sub-step with the isotropic 19-point Laplacian; a plane beyond a
 // wall holds 2 T_w - T of the wall plane (halfway ghost).
 template <typename R>
-__global__ void k_tsub3d_iso(Geom g, Phys<R> p, const R* __restrict__ Tin, R* __restrict__ Tout)
+__global__ void k_tsub3d_iso(Geom g, Phys<R> p, const R* Tin, R* Tout)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
+    chain_next();
+    chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch;
     const int zs = ny * pitch;                   // 32-bit offsets: Q * padded sites < 2^31 (checked at creation)
@@ -569,11 +573,8 @@ template <typename R>
 cudaError_t launch_tsub3d(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, cudaStream_t s)
 {
     dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
-    if (g.stencil == LF_STENCIL_ISOTROPIC)
-        k_tsub3d_iso<R><<<grd, blk, 0, s>>>(g, p, Tin, Tout);
-    else
-        k_tsub3d<R><<<grd, blk, 0, s>>>(g, p, Tin, Tout);
-    return cudaGetLastError();
+    return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub3d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
+                                             : launch_chained(k_tsub3d<R>, grd, blk, 0, s, g, p, Tin, Tout);
 }
 
 template cudaError_t launch_step3d<float>(const Geom&, const Phys<float>&, const StepIO<float>&, bool, cudaStream_t);

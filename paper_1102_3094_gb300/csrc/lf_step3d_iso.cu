@@ -80,6 +80,7 @@ __global__ void __launch_bounds__(Force3Iso<R, TX, TY>::NTH, MINB) k_force3d_iso
         if (q < W3) colmap[q] = wrap_s(x0 - 3 + q, nx);
         else rowmap[q - W3] = wrap_s(y0 - 3 + (q - W3), ny);
     }
+    chain_wait();
     __syncthreads();
     const int col_off = rowmap[cy + 1] * pitch + colmap[cx + 1];
     const int c3 = (cy + 1) * W3 + cx + 1;
@@ -205,6 +206,7 @@ __global__ void __launch_bounds__(Force3Iso<R, TX, TY>::NTH, MINB) k_force3d_iso
         iter(k + 1, std::integral_constant<int, 1>{});
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -302,6 +304,7 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
         if (q < W3) colmap[q] = wrap_s(x0 - 3 + q, nx);
         else rowmap[q - W3] = wrap_s(y0 - 3 + (q - W3), ny);
     }
+    chain_wait();
     __syncthreads();
     const int col_off = rowmap[cy + 1] * pitch + colmap[cx + 1];
     const int c3 = (cy + 1) * W3 + cx + 1;
@@ -478,6 +481,7 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
         iter(j + 1, I1{}, GEN{});
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -556,6 +560,7 @@ __global__ void __launch_bounds__(256) k_phi3d_isoz(Geom g, Phys<R> p, StepIO<R>
     Slide19<R> smu, sT, sgx, sgy, sgz;
     R Tc1 = R(0);                                           // own T of plane k - 1
     bool bad = false;
+    chain_wait();
     fetch(za - 1);
     put(za - 1);
     for (int k = za - 1; k <= zb; ++k) {
@@ -596,6 +601,7 @@ __global__ void __launch_bounds__(256) k_phi3d_isoz(Geom g, Phys<R> p, StepIO<R>
         Tc1 = Tck;
         if (k < zb) put(k + 1);                             // slot of plane k - 1, read by nobody now
     }
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -655,6 +661,7 @@ __global__ void __launch_bounds__(256) k_phi3d_isoa(Geom g, Phys<R> p, StepIO<R>
     Slide19<R> smu, sT, sgx, sgy, sgz;
     R Tc1 = R(0);
     bool bad = false;
+    chain_wait();
     fetch(za - 1);
     fetch(za);
     for (int k = za - 1; k <= zb; ++k) {
@@ -714,6 +721,7 @@ __global__ void __launch_bounds__(256) k_phi3d_isoa(Geom g, Phys<R> p, StepIO<R>
         Tc1 = Tck;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -734,8 +742,7 @@ cudaError_t launch_force_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
-    kern<<<grid, P3::NTH, P3::BYTES, s>>>(g, p, io, Hz);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, P3::NTH, P3::BYTES, s, g, p, io, Hz);
 }
 
 template <int TX, int TY>
@@ -755,8 +762,7 @@ cudaError_t launch_force_iso_x2(const Geom& g, const Phys<float>& p, const StepI
     }
     if (H > g.nz) H = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + 2 * H - 1) / (2 * H));
-    kern<<<grid, P3::NTH, P3::BYTES, s>>>(g, p, io, H);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, P3::NTH, P3::BYTES, s, g, p, io, H);
 }
 
 }  // namespace
@@ -787,15 +793,13 @@ cudaError_t launch_phi3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
         static unsigned long long attr_done = 0;
         const cudaError_t e = raise_smem_limit(k_phi3d_isoa<R>, (int)bytes, &attr_done);
         if (e != cudaSuccess) return e;
-        k_phi3d_isoa<R><<<gc, 256, bytes, s>>>(g, p, io, zc);
-        return cudaGetLastError();
+        return launch_chained(k_phi3d_isoa<R>, gc, 256, bytes, s, g, p, io, zc);
     }
     constexpr size_t bytes = sizeof(R) * 2 * kIsoNF * kIsoTA;
     static unsigned long long attr_done = 0;
     const cudaError_t e = raise_smem_limit(k_phi3d_isoz<R>, (int)bytes, &attr_done);
     if (e != cudaSuccess) return e;
-    k_phi3d_isoz<R><<<gc, 256, bytes, s>>>(g, p, io, zc);
-    return cudaGetLastError();
+    return launch_chained(k_phi3d_isoz<R>, gc, 256, bytes, s, g, p, io, zc);
 }
 
 template cudaError_t launch_force3d_iso<float>(const Geom&, const Phys<float>&, const StepIO<float>&, cudaStream_t);

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(Force3<R, TX, TY>::NTH) k_force3d(Geom g, Phys
         if (q < W3) colmap[q] = wrap_s(x0 - 3 + q, nx);
         else rowmap[q - W3] = wrap_s(y0 - 3 + (q - W3), ny);
     }
+    chain_wait();
     __syncthreads();
     // storage offset of this column inside a plane (wrapped)
     const int col_off = rowmap[cy + 1] * pitch + colmap[cx + 1];
@@ -197,6 +198,7 @@ __global__ void __launch_bounds__(Force3<R, TX, TY>::NTH) k_force3d(Geom g, Phys
         Tq3 = Tq2; Tq2 = Tq1; Tq1 = Tq0; Tq0 = Tnext;
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -253,6 +255,7 @@ __global__ void __launch_bounds__(Force3x2<TX, TY>::NTH, 2) k_force3d_x2(Geom g,
         if (q < W3) colmap[q] = wrap_s(x0 - 3 + q, nx);
         else rowmap[q - W3] = wrap_s(y0 - 3 + (q - W3), ny);
     }
+    chain_wait();
     __syncthreads();
     const int col_off = rowmap[cy + 1] * pitch + colmap[cx + 1];
     const int c3 = (cy + 1) * W3 + cx + 1;
@@ -394,6 +397,7 @@ __global__ void __launch_bounds__(Force3x2<TX, TY>::NTH, 2) k_force3d_x2(Geom g,
         iter(j + 3, std::integral_constant<int, 3>{});
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    chain_next();
     if (__any_sync(0xffffffffu, bad) && (t & 31) == 0) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -405,6 +409,8 @@ __global__ void __launch_bounds__(128) k_lb3d(Geom g, Phys<R> p, StepIO<R> io)
 {
     using L = D3Q19;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, z = blockIdx.z;
+    chain_next();                                // many waves of small blocks: the next pass fills the last one
+    chain_wait();
     if (x >= g.nx) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch, walls = g.walls;
     const int plane = (int)g.plane, zs = ny * pitch;   // 32-bit offsets: Q * padded sites < 2^31 (checked at creation)
@@ -474,6 +480,7 @@ __global__ void __launch_bounds__(256) k_phi3d(Geom g, Phys<R> p, StepIO<R> io, 
 {
     const int x = blockIdx.x * 32 + (threadIdx.x & 31), y = blockIdx.y * 8 + (threadIdx.x >> 5);
     const int za = blockIdx.z * zc, zb = min(za + zc, g.nz);
+    chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch, walls = g.walls;
     const int64_t zs = (int64_t)ny * pitch;
@@ -559,6 +566,7 @@ __global__ void __launch_bounds__(256) k_phi3d(Geom g, Phys<R> p, StepIO<R> io, 
         gz_d = gz_c; gz_c = gz_u;
         nb = nxt;
     }
+    chain_next();
     if (bad) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -579,8 +587,7 @@ cudaError_t launch_force(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
-    kern<<<grid, P3::NTH, P3::BYTES, s>>>(g, p, io, Hz);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, P3::NTH, P3::BYTES, s, g, p, io, Hz);
 }
 
 template <int TX, int TY>
@@ -601,8 +608,7 @@ cudaError_t launch_force_x2(const Geom& g, const Phys<float>& p, const StepIO<fl
     }
     if (H > g.nz) H = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + 2 * H - 1) / (2 * H));
-    kern<<<grid, P3::NTH, P3::BYTES, s>>>(g, p, io, H);
-    return cudaGetLastError();
+    return launch_chained(kern, grid, P3::NTH, P3::BYTES, s, g, p, io, H);
 }
 
 }  // namespace
@@ -627,16 +633,14 @@ template <typename R>
 cudaError_t launch_lb3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cudaStream_t s)
 {
     dim3 grid((g.nx + 127) / 128, g.ny, g.nz);
-    k_lb3d<R><<<grid, 128, 0, s>>>(g, p, io);
-    return cudaGetLastError();
+    return launch_chained(k_lb3d<R>, grid, 128, 0, s, g, p, io);
 }
 
 template <typename R>
 cudaError_t launch_phi3d_compact(const Geom& g, const Phys<R>& p, const StepIO<R>& io, int zc, cudaStream_t s)
 {
     dim3 gc((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
-    k_phi3d<R><<<gc, 256, 0, s>>>(g, p, io, zc);
-    return cudaGetLastError();
+    return launch_chained(k_phi3d<R>, gc, 256, 0, s, g, p, io, zc);
 }
 
 #define LF_INST(R)                                                                                              \
