@@ -6,8 +6,9 @@
 //   A  mu and F = -d_a P_ab (Eqs. chem, ff): k_force3d_iso (one lane, FP32
 //      and FP64) or k_force3d_iso_x2 (two z-lanes in packed FP32x2);
 //   C  phi(t+1) = phi - div(phi u) + Gamma lap(mu) (Eq. massdiff) and the
-//      first temperature sub-step: k_phi3d_isoz (fields staged through
-//      registers) or k_phi3d_isoa (raw fields staged by cp.async).
+//      first temperature sub-step in FP64: k_phi3d_isoz (fields staged through
+//      registers) or k_phi3d_isoa (raw fields staged by cp.async); in FP32 the
+//      pass is lf_step3d_phi.cu.
 // Pass B (collision and streaming) is the same for both stencils.  The wall
 // rules are those of the compact passes: phi, T and every derived scalar
 // even about the half-way planes, the wall-normal flux odd, T with its
@@ -784,8 +785,7 @@ cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>&
     }
 }
 
-template <typename R>
-cudaError_t launch_phi3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& io, int zc, cudaStream_t s)
+cudaError_t launch_phi3d_iso(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s)
 {
     dim3 gc((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     if ((g.tune >> 28) & 1) {                           // param bit 28: the raw fields staged by cp.async
@@ -796,6 +796,7 @@ cudaError_t launch_phi3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
         return launch_chained(k_phi3d_isoa<R>, gc, 256, bytes, s, g, p, io, zc);
     }
     constexpr size_t bytes = sizeof(R) * 2 * kIsoNF * kIsoTA;
+    using R = double;
     static unsigned long long attr_done = 0;
     const cudaError_t e = raise_smem_limit(k_phi3d_isoz<R>, (int)bytes, &attr_done);
     if (e != cudaSuccess) return e;
@@ -804,7 +805,5 @@ cudaError_t launch_phi3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
 
 template cudaError_t launch_force3d_iso<float>(const Geom&, const Phys<float>&, const StepIO<float>&, cudaStream_t);
 template cudaError_t launch_force3d_iso<double>(const Geom&, const Phys<double>&, const StepIO<double>&, cudaStream_t);
-template cudaError_t launch_phi3d_iso<float>(const Geom&, const Phys<float>&, const StepIO<float>&, int, cudaStream_t);
-template cudaError_t launch_phi3d_iso<double>(const Geom&, const Phys<double>&, const StepIO<double>&, int, cudaStream_t);
 
 }  // namespace lf

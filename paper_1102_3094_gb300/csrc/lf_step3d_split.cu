@@ -7,7 +7,8 @@
 //      streaming with halfway bounce-back (Eqs. moment, evoleqn,
 //      latticeforceterm), one thread per site; writes u(t);
 //   C  k_phi3d: phi(t+1) = phi - div(phi u) + Gamma lap(mu) (Eq. massdiff)
-//      and the first temperature sub-step, one thread per site.
+//      and the first temperature sub-step, one thread per column (FP64; in
+//      FP32 the pass is lf_step3d_phi.cu, four sites per thread).
 // mu, F and u pass through the context's aux planes.  The arithmetic per site
 // is that of the fused plane march (lf_step3d.cu), with the same wall rules:
 // even reflection of phi, T and every derived scalar about the half-way
@@ -636,8 +637,8 @@ cudaError_t launch_lb3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cu
     return launch_chained(k_lb3d<R>, grid, 128, 0, s, g, p, io);
 }
 
-template <typename R>
-cudaError_t launch_phi3d_compact(const Geom& g, const Phys<R>& p, const StepIO<R>& io, int zc, cudaStream_t s)
+cudaError_t launch_phi3d_compact(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s)
+    using R = double;
 {
     dim3 gc((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     return launch_chained(k_phi3d<R>, gc, 256, 0, s, g, p, io, zc);
@@ -645,8 +646,7 @@ cudaError_t launch_phi3d_compact(const Geom& g, const Phys<R>& p, const StepIO<R
 
 #define LF_INST(R)                                                                                              \
     template cudaError_t launch_force3d_compact<R>(const Geom&, const Phys<R>&, const StepIO<R>&, cudaStream_t); \
-    template cudaError_t launch_lb3d<R>(const Geom&, const Phys<R>&, const StepIO<R>&, cudaStream_t);           \
-    template cudaError_t launch_phi3d_compact<R>(const Geom&, const Phys<R>&, const StepIO<R>&, int, cudaStream_t);
+    template cudaError_t launch_lb3d<R>(const Geom&, const Phys<R>&, const StepIO<R>&, cudaStream_t);
 LF_INST(float)
 LF_INST(double)
 #undef LF_INST

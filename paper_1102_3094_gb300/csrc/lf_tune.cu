@@ -77,7 +77,7 @@ std::vector<std::pair<int, int>> candidates(const lf_ctx* c)
             const int* sels = c->prec == LF_FP32 ? sels32 : sels64;
             const int nsel = c->prec == LF_FP32 ? 4 : 1;
             const int lanes[] = {0, 48, 64, 96, 128, 192};   // planes per lane of the packed form
-            for (int phi_form = 0; phi_form < 2; ++phi_form)  // phi pass: register-staged, cp.async-staged (bit 28)
+            for (int phi_form = 0; phi_form < (c->prec == LF_FP64 ? 2 : 1); ++phi_form)  // FP64 phi pass: register-staged, cp.async-staged (bit 28)
                 for (int i = 0; i < nsel; ++i) {
                     const int base = (phi_form << 28) | (zc << 20) | (sels[i] << 16);
                     if (sels[i] == 4) {
