@@ -263,19 +263,21 @@ int lf_load(lf_ctx* ctx, const char* path);
  *     isotropic stencils the two segments are the lower and upper halves of a
  *     pair, both marching upwards, with sliding row sums;
  *   LF_VARIANT_SPLIT3 (3D default): three passes per step -- mu and F by a
- *     plane march ((param & 0xFFFF) = planes per segment, 0 = automatic),
- *     then collision and streaming, then the phi and T updates by a column
- *     march over (param >> 20) & 255 planes per segment (0 = 16); mu, F and
- *     u pass through the context's derived-field planes.  (param >> 16) & 15
- *     selects the force pass's form: with the compact stencils, in FP32, 0 =
- *     two segments in the lanes of packed FP32x2 arithmetic, 1 / 2 = one lane
- *     on 60x4 / 28x12 tiles; with the isotropic stencils (both passes as
- *     column marches with sliding plane sums), 0 = one lane on 28x12 tiles
- *     (FP32: two CTAs per SM), 1 = on 28x28 tiles, 3 = on 28x12 tiles at one
- *     CTA per SM, 4 = two segments in packed FP32x2 lanes (1, 3 and 4 in FP32
- *     only; FP64 takes 0); with the isotropic stencils bit 28 selects the
- *     phi pass that stages its raw fields by cp.async.  For 3D contexts every
- *     other variant runs the fused plane march (param = planes per segment).
+ *     plane march ((param & 0xFFFF) = planes per segment, 0 = chosen from the
+ *     lattice sizes and the SM count), then collision and streaming, then the
+ *     phi and T updates by a column march over (param >> 20) & 255 planes per
+ *     segment (0 = automatic); mu, F and u pass through the context's
+ *     derived-field planes.  (param >> 16) & 15 selects the force pass's form:
+ *     with the compact stencils, in FP32, 0 = two segments in the lanes of
+ *     packed FP32x2 arithmetic, 1 / 2 = one lane on 60x4 / 28x12 tiles; with
+ *     the isotropic stencils (both passes as column marches with sliding plane
+ *     sums), 0 = one lane on 28x12 tiles (FP32: two CTAs per SM, and the form
+ *     4 when the planes per segment are automatic too), 1 = on 28x28 tiles,
+ *     3 = on 28x12 tiles at one CTA per SM, 4 = two segments in packed FP32x2
+ *     lanes (1, 3 and 4 in FP32 only; FP64 takes 0); with the isotropic
+ *     stencils bit 28 selects, in FP64, the phi pass that stages its raw
+ *     fields by cp.async.  For 3D contexts every other variant runs the fused
+ *     plane march (param = planes per segment).
  * Returns LF_EINVAL for an unknown variant or a negative param. */
 #define LF_VARIANT_MARCH  0
 #define LF_VARIANT_TILE   1

@@ -40,5 +40,34 @@ __device__ __forceinline__ void cp_async_s(void* dst, const void* src)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
 
+// Planes per segment (or per lane of a two-lane segment: `lanes` = 2) of a
+// column march over `tiles` columns of a CTA, `lag` planes longer than its
+// segment, `res` CTAs resident per SM.  The march of a CTA takes about as
+// long as it has planes, so the time is the number of rounds of resident CTAs
+// times (planes + lag); a last round that leaves every SM at most one of two
+// places runs at 0.6 of a full one (an SM's issue rate is then shared by half
+// the CTAs).  The number of segments with the least of that wins; few planes
+// per segment on small lattices, where everything fits in one round and only
+// the length of the march counts.  Over ten lattices from 32 x 32 x 256 to
+// 384^3 and both stencils the packed force pass comes within 4 % (48 x 380 x
+// 90: 13 %) of its best height; segments of at least 16 planes, the rule
+// before, cost 64^3 29.5 us instead of 15.0 (compact) and 32 x 32 x 256 29.2
+// instead of 18.2.
+inline int march3_planes(int64_t tiles, int nz, int lanes, int lag, int res, int sms)
+{
+    int best = nz;
+    double best_cost = 1e300;
+    for (int k = 1; k * lanes <= 2 * nz && k <= 4096; ++k) {
+        const int H = (nz + k * lanes - 1) / (k * lanes);
+        const int64_t ctas = tiles * ((nz + H * lanes - 1) / (H * lanes));
+        const int64_t full = ctas / (res * (int64_t)sms), left = ctas - full * res * sms;
+        const double rounds = (double)full + (left == 0 ? 0.0 : (res == 2 && left <= sms ? 0.6 : 1.0));
+        const double cost = rounds * (H + lag);
+        if (cost < best_cost) { best_cost = cost; best = H; }
+        if (H == 1) break;
+    }
+    return best;
+}
+
 }  // namespace
 }  // namespace lf

@@ -215,7 +215,10 @@ __global__ void __launch_bounds__(Force3Iso<R, TX, TY>::NTH, MINB) k_force3d_iso
 // marches planes [z0, z0 + H), lane .y planes [z0 + H, z0 + 2H) (shorter or
 // empty at the top of the lattice), with the stages and lags of
 // k_force3d_iso, float2 shared planes (one 64-bit load brings a neighbour of
-// both lanes) and packed FP32x2 arithmetic throughout.
+// both lanes) and packed FP32x2 arithmetic throughout.  The products are
+// grouped as the compiler groups the one-lane form's, so both give the same
+// bits (pinned by a test): isotropic runs after a deep quench amplify rounding
+// differences ten thousandfold in 600 steps.
 template <int TX, int TY>
 struct Force3IsoX2 {
     static constexpr int CW = TX + 4, CH = TY + 4, NTH = CW * CH;
@@ -245,8 +248,8 @@ __device__ __forceinline__ Plane plane(const float2* a, int c, float2 ac)
     r.l = fma2(v2(-24.f), ac, fma2(v2(2.f), cross, add2(add2(ne, nw), add2(se, sw))));
     r.ax = sub2(e, w);
     r.ay = sub2(n, so);
-    r.gx = fma2(v2(2.f), r.ax, add2(sub2(ne, nw), sub2(se, sw)));
-    r.gy = fma2(v2(2.f), r.ay, add2(sub2(ne, se), sub2(nw, sw)));
+    r.gx = add2(fma2(v2(2.f), r.ax, sub2(ne, nw)), sub2(se, sw));
+    r.gy = add2(fma2(v2(2.f), r.ay, sub2(ne, se)), sub2(nw, sw));
     return r;
 }
 struct Slide {
@@ -366,7 +369,6 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
         if constexpr (FULL) fetch_at(ba + zs, bb + zs, PAR ^ 1);
-        else fetch(j + 1, PAR ^ 1);
 
         // phi plane j: psi and grad phi at j - 1 (every column)
         float2 phk, psk, dxk, dyk, dzk;
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
                 const float2 av = mul2(sub2(Tc, v2(p.Tc)), v2(p.inv_Tc));
                 const float2 phsq = mul2(ph, ph);
                 if (own && (FULL || r2 >= 0)) {
-                    const float2 mu = fma2(v2(p.c), lam, fma2(v2(-p.kappa), psi, mul2(ph, fma2(v2(p.b), phsq, av))));
+                    const float2 mu = fma2(v2(p.c), lam, fma2(v2(-p.kappa), psi, fma2(mul2(mul2(v2(p.b), ph), ph), ph, mul2(av, ph))));
                     if constexpr (FULL) {
                         bad |= !isfinite(mu.x) || !isfinite(mu.y);
                         io.mu[ba - zs3 + own_off] = mu.x;
@@ -401,18 +403,20 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
                 }
                 if (hyd) {
                     const float2 d0 = dx2, d1 = dy2, d2 = dz2;
-                    const float2 gp2 = fma2(d0, d0, fma2(d1, d1, mul2(d2, d2)));
-                    const float2 gpgs = fma2(d0, s0, fma2(d1, s1, mul2(d2, s2)));
-                    float2 iso = mul2(phsq, fma2(v2(0.75f * p.b), phsq, mul2(half, av)));
-                    iso = fma2(v2(-p.kappa), fma2(half, gp2, mul2(ph, psi)), iso);
-                    iso = fma2(v2(p.c), add2(fma2(ph, lam, mul2(half, mul2(psi, psi))), gpgs), iso);
+                    const float2 gp2 = fma2(d2, d2, fma2(d0, d0, mul2(d1, d1)));
+                    float2 iso = fma2(mul2(v2(0.75f * p.b), phsq), phsq, mul2(mul2(av, phsq), half));
+                    iso = fma2(v2(-p.kappa), fma2(ph, psi, mul2(half, gp2)), iso);
+                    float2 q = fma2(mul2(half, psi), psi, mul2(ph, lam));
+                    q = fma2(d2, s2, fma2(d1, s1, fma2(d0, s0, q)));
+                    iso = fma2(v2(p.c), q, iso);
                     float2* P = sP + (PAR ^ 1) * 6 * A2;
-                    nxz = fma2(k_, mul2(d0, d2), mul2(mc, fma2(d0, s2, mul2(d2, s0))));
-                    nyz = fma2(k_, mul2(d1, d2), mul2(mc, fma2(d1, s2, mul2(d2, s1))));
-                    nzz = fma2(k_, mul2(d2, d2), fma2(m2c, mul2(d2, s2), iso));
-                    P[0 * A2 + c2] = fma2(k_, mul2(d0, d0), fma2(m2c, mul2(d0, s0), iso));
-                    P[1 * A2 + c2] = fma2(k_, mul2(d0, d1), mul2(mc, fma2(d0, s1, mul2(d1, s0))));
-                    P[2 * A2 + c2] = fma2(k_, mul2(d1, d1), fma2(m2c, mul2(d1, s1), iso));
+                    const float2 kd0 = mul2(k_, d0), kd1 = mul2(k_, d1), kd2 = mul2(k_, d2);
+                    nxz = fma2(kd0, d2, mul2(mc, fma2(d2, s0, mul2(d0, s2))));
+                    nyz = fma2(kd1, d2, mul2(mc, fma2(d2, s1, mul2(d1, s2))));
+                    nzz = fma2(mul2(m2c, d2), s2, fma2(kd2, d2, iso));
+                    P[0 * A2 + c2] = fma2(mul2(m2c, d0), s0, fma2(kd0, d0, iso));
+                    P[1 * A2 + c2] = fma2(kd0, d1, mul2(mc, fma2(d1, s0, mul2(d0, s1))));
+                    P[2 * A2 + c2] = fma2(mul2(m2c, d1), s1, fma2(kd1, d1, iso));
                     P[3 * A2 + c2] = nxz;
                     P[4 * A2 + c2] = nyz;
                     P[5 * A2 + c2] = nzz;
@@ -732,14 +736,14 @@ cudaError_t launch_force_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     using P3 = Force3Iso<R, TX, TY>;
     auto kern = k_force3d_iso<R, TX, TY, MINB>;
     static unsigned long long attr_done = 0;      // per instantiation and device
-    const cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
+    cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
     const int tiles = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
     int Hz = (g.tune & 0xFFFF) > 0 ? (g.tune & 0xFFFF) : 0;
-    if (Hz <= 0) {   // about eight waves of the resident CTAs, segments of at least 16 planes
-        const int want = (8 * MINB * 152 + tiles - 1) / tiles;
-        Hz = (g.nz + want - 1) / want;
-        if (Hz < 16) Hz = 16;
+    if (Hz <= 0) {
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        Hz = march3_planes(tiles, g.nz, 1, 8, MINB, sms);
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
@@ -752,14 +756,14 @@ cudaError_t launch_force_iso_x2(const Geom& g, const Phys<float>& p, const StepI
     using P3 = Force3IsoX2<TX, TY>;
     auto kern = k_force3d_iso_x2<TX, TY>;
     static unsigned long long attr_done = 0;      // per instantiation and device
-    const cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
+    cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
     const int tiles = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
     int H = (g.tune & 0xFFFF) > 0 ? (g.tune & 0xFFFF) : 0;     // planes per lane
-    if (H <= 0) {   // about eight waves of one CTA per SM, lanes of at least 16 planes
-        const int want = (8 * 152 + tiles - 1) / tiles;
-        H = (g.nz + 2 * want - 1) / (2 * want);
-        if (H < 16) H = 16;
+    if (H <= 0) {
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        H = march3_planes(tiles, g.nz, 2, 8, 1, sms);
     }
     if (H > g.nz) H = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + 2 * H - 1) / (2 * H));
@@ -773,8 +777,13 @@ cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>&
 {
     // (param >> 16) & 15: 0 = one lane on 28x12 tiles (FP32: two CTAs per SM),
     // 1 = one lane on 28x28 tiles, 3 = one lane on 28x12 tiles at one CTA per
-    // SM, 4 = two z-lanes in packed FP32x2 on 28x12 tiles (1, 3, 4: FP32 only)
-    const int sel = (g.tune >> 16) & 15;
+    // SM, 4 = two z-lanes in packed FP32x2 on 28x12 tiles (1, 3, 4: FP32 only).
+    // With no planes per segment given either, FP32 takes the packed form: it
+    // is the fastest from 64^3 up (64^3: 18.9 us against 29.7 for one lane with
+    // segments of 16 planes, 128^3 63 / 66, 250 x 243 x 190 241 / 284, 384^3
+    // 937 / 1138).
+    int sel = (g.tune >> 16) & 15;
+    if (sizeof(R) == 4 && (g.tune & 0xFFFFF) == 0) sel = 4;
     if constexpr (sizeof(R) == 4) {
         return sel == 1 ? launch_force_iso<R, 28, 28, 1>(g, p, io, s)
              : sel == 3 ? launch_force_iso<R, 28, 12, 1>(g, p, io, s)
@@ -787,6 +796,7 @@ cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>&
 
 cudaError_t launch_phi3d_iso(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s)
 {
+    using R = double;
     dim3 gc((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     if ((g.tune >> 28) & 1) {                           // param bit 28: the raw fields staged by cp.async
         constexpr size_t bytes = sizeof(R) * 3 * kIsoNR * kIsoTA;
@@ -796,7 +806,6 @@ cudaError_t launch_phi3d_iso(const Geom& g, const Phys<double>& p, const StepIO<
         return launch_chained(k_phi3d_isoa<R>, gc, 256, bytes, s, g, p, io, zc);
     }
     constexpr size_t bytes = sizeof(R) * 2 * kIsoNF * kIsoTA;
-    using R = double;
     static unsigned long long attr_done = 0;
     const cudaError_t e = raise_smem_limit(k_phi3d_isoz<R>, (int)bytes, &attr_done);
     if (e != cudaSuccess) return e;

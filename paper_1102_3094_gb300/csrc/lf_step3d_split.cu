@@ -577,14 +577,14 @@ cudaError_t launch_force(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     using P3 = Force3<R, TX, TY>;
     auto kern = k_force3d<R, TX, TY>;
     static unsigned long long attr_done = 0;      // per instantiation and device
-    const cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
+    cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
     const int tiles = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
     int Hz = (g.tune & 0xFFFF) > 0 ? (g.tune & 0xFFFF) : 0;
-    if (Hz <= 0) {   // about eight waves of two CTAs per SM, segments of at least 16 planes
-        const int want = (8 * 2 * 152 + tiles - 1) / tiles;
-        Hz = (g.nz + want - 1) / want;
-        if (Hz < 16) Hz = 16;
+    if (Hz <= 0) {
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        Hz = march3_planes(tiles, g.nz, 1, 5, sizeof(R) == 4 ? 2 : 1, sms);
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
@@ -597,15 +597,14 @@ cudaError_t launch_force_x2(const Geom& g, const Phys<float>& p, const StepIO<fl
     using P3 = Force3x2<TX, TY>;
     auto kern = k_force3d_x2<TX, TY>;
     static unsigned long long attr_done = 0;      // per instantiation and device
-    const cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
+    cudaError_t e = raise_smem_limit(kern, (int)P3::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
     const int tiles = ((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
     int H = (g.tune & 0xFFFF) > 0 ? (g.tune & 0xFFFF) : 0;     // planes per lane
-    if (H <= 0) {   // about eight CTAs per SM (two resident), lanes of at least 16 planes
-        const int want = (8 * 152 + tiles - 1) / tiles;
-        H = (g.nz + 2 * want - 1) / (2 * want);
-        if (H < 16) H = 16;
-        H += (6 - H % 4) % 4;   // H + 6 iterations: whole trips of four
+    if (H <= 0) {
+        int sms = 0;
+        if ((e = device_sms(&sms)) != cudaSuccess) return e;
+        H = march3_planes(tiles, g.nz, 2, 6, 2, sms);
     }
     if (H > g.nz) H = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + 2 * H - 1) / (2 * H));
@@ -638,8 +637,8 @@ cudaError_t launch_lb3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cu
 }
 
 cudaError_t launch_phi3d_compact(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s)
-    using R = double;
 {
+    using R = double;
     dim3 gc((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + zc - 1) / zc);
     return launch_chained(k_phi3d<R>, gc, 256, 0, s, g, p, io, zc);
 }

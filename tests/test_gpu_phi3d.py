@@ -49,3 +49,23 @@ def test_nonfinite_site_is_seen_and_padding_is_not():
     sim.step(1)
     assert sim.diag()["rc"] == lf.LF_ENONFINITE
     sim.close()
+
+
+@pytest.mark.parametrize("opt", [dict(), dict(walls=0), dict(t_wall_mode=1), dict(hydro=0)],
+                         ids=["layers", "periodic", "halfway", "nohydro"])
+@pytest.mark.parametrize("shape", [(32, 20, 17), (29, 13, 40), (61, 25, 33)], ids=lambda s: "x".join(map(str, s)))
+def test_packed_and_one_lane_force_passes_give_the_same_bits(shape, opt):
+    """The isotropic force pass on two packed lanes (the automatic choice) against one lane: three steps, every bit."""
+    from paper_1102_3094_gb300 import lf
+
+    out = []
+    for param in (0, 5, (4 << 16) | 7):           # automatic (packed), one lane of 5 planes, packed lanes of 7
+        sim = lf.Lattice(d=3, nx=shape[0], ny=shape[1], nz=shape[2], precision="fp32", stencil="isotropic", xi=0.1,
+                         tau=3.0, phi_amp=0.4, **opt)
+        sim.set_variant("split3", param)
+        sim.step(3)
+        out.append([sim.get(k) for k in ("phi", "T", "pop")])
+        sim.close()
+    for other in out[1:]:
+        for a, b in zip(out[0], other):
+            np.testing.assert_array_equal(a, b)
