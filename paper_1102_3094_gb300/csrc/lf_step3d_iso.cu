@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(Force3IsoX2<TX, TY>::NTH, 1) k_force3d_iso_x2(
         asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
         if constexpr (FULL) fetch_at(ba + zs, bb + zs, PAR ^ 1);
+        else fetch(j + 1, PAR ^ 1);
 
         // phi plane j: psi and grad phi at j - 1 (every column)
         float2 phk, psk, dxk, dyk, dzk;
