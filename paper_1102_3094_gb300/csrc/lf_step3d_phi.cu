@@ -125,7 +125,6 @@ __global__ void __launch_bounds__(128) k_phi3d_q(Geom g, Phys<float> p, StepIO<f
     const int row = q.y * pitch;
     const int rl = (q.y == 0 ? g.ny - 1 : q.y - 1) * pitch, rr = (q.y + 1 == g.ny ? 0 : q.y + 1) * pitch;
     const float half = 0.5f;
-    chain_next();
     chain_wait();
     int o = z_below(za, nz, walls) * zs + row;
     Q4 mu_d = q.load(io.mu + o), T_d = q.load(io.T_in + o), gz_d{}, gz_c{}, ph_c;
@@ -189,6 +188,7 @@ __global__ void __launch_bounds__(128) k_phi3d_q(Geom g, Phys<float> p, StepIO<f
         gz_d = gz_c; gz_c = gz_u;
         ph_c = ph_u;
     }
+    chain_next();
     if (bad) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
@@ -222,7 +222,6 @@ __global__ void __launch_bounds__(128, 3) k_phi3d_iso_q(Geom g, Phys<float> p, S
     const int row = q.y * pitch;
     const int rl = (q.y == 0 ? g.ny - 1 : q.y - 1) * pitch, rr = (q.y + 1 == g.ny ? 0 : q.y + 1) * pitch;
     const bool halfway = walls && g.t_mode == LF_TWALL_HALFWAY;
-    chain_next();
     chain_wait();
     // sums of the open centre and the last plane's parts, per site
     float ml[4], ms[4], tl[4], ts[4];            // lap mu, lap T
@@ -323,6 +322,7 @@ __global__ void __launch_bounds__(128, 3) k_phi3d_iso_q(Geom g, Phys<float> p, S
         T1 = tc;
         ph1 = pc;
     }
+    chain_next();
     if (bad) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
