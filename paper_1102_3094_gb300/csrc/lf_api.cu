@@ -196,10 +196,12 @@ int do_steps(lf_ctx* c, int64_t n)
             const int rc = t_implicit_step<R>(c, c->params.xi, c->walls.T_w);
             if (rc != LF_OK) return rc;
         } else if (ph.t_update) {
-            for (int s = 1; s < c->nsub; ++s) {
-                if (launch_tsub<R>(c->g, ph, (const R*)c->T[c->tcur], (R*)c->T[c->tcur ^ 1], c->stream) != cudaSuccess)
+            for (int left = c->nsub - 1; left > 0;) {
+                const int n = tsub_fused<R>(c->g, left);
+                if (launch_tsub<R>(c->g, ph, (const R*)c->T[c->tcur], (R*)c->T[c->tcur ^ 1], n, c->stream) != cudaSuccess)
                     return LF_ECUDA;
                 c->tcur ^= 1;
+                left -= n;
             }
         }
         c->step += 1;

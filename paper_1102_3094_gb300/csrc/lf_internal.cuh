@@ -129,8 +129,12 @@ cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>&
 cudaError_t launch_phi3d_iso(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s);
 template <typename R>
 cudaError_t launch_tsub3d(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, cudaStream_t s);
+// extra temperature sub-steps: how many of the `left` remaining ones the next
+// launch takes, and that launch
 template <typename R>
-cudaError_t launch_tsub(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, cudaStream_t s);
+int tsub_fused(const Geom& g, int left);
+template <typename R>
+cudaError_t launch_tsub(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, int n, cudaStream_t s);
 template <typename R>
 cudaError_t launch_init(const Geom& g, uint64_t seed, double amp, double T0, double T_w,
                         int quench, R* phi, R* T, cudaStream_t s);
@@ -236,20 +240,31 @@ inline cudaError_t device_sms(int* sms)
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// `spread` > 0: the share of the L1 that becomes shared memory is what `spread`
+// CTAs of this kernel need, not what most would.
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args)
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, int spread, cudaStream_t s, const A&... args)
 {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    const size_t want = spread * (smem + 1024), all = 228 * 1024;      // 1 KB per CTA is the system's
+    at[1].val.sharedMemCarveout = want < all ? (unsigned)((want * 100 + all - 1) / all) : 100;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = spread > 0 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args)
+{
+    return launch_chained(kern, grid, block, smem, 0, s, args...);
 }
 
 }  // namespace lf

@@ -41,8 +41,10 @@
 #include "lf_march2d_iso.cuh"
 #include "lf_march2d_x2.cuh"
 #include "lf_tile2d.cuh"
+#include "lf_tsub2d.cuh"
 
 namespace lf {
+
 
 namespace {
 
@@ -96,6 +98,20 @@ __global__ void __launch_bounds__(NT, MINB) k_march2d_x2(Geom g, Phys<float> p, 
     chain_next();
 }
 
+// CTAs per SM to leave room for: what an even spread of a march's grid gives
+// when that is below the `most` that fit, else 0 (no preference).  A grid that
+// is let in while its predecessor drains would otherwise fill the SMs that are
+// free first: 2999 x 1777 after its temperature sub-steps 147 us a step, 114
+// with two CTAs per SM.  FP64 marches, bound by their pipe, take at most two
+// (512^2: 242 -> 174 us, 1024^2 the same).
+template <typename R>
+int spread_of(dim3 grid, int sms, int most = sizeof(R) == 4 ? 3 : 2)
+{
+    const int64_t k = ((int64_t)grid.x * grid.y + sms - 1) / sms;
+    if (sizeof(R) == 8) return k < most ? (int)k : most;
+    return k < most ? (int)k : 0;
+}
+
 template <int NT, int D, bool HYDRO, int MINB>
 cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, cudaStream_t s)
 {
@@ -110,7 +126,7 @@ cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<fl
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -125,7 +141,7 @@ cudaError_t launch_march(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, H);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<R>(grid, sms), s, g, p, io, H);
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
@@ -142,7 +158,7 @@ cudaError_t launch_march_iso_x2(const Geom& g, const Phys<float>& p, const StepI
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -157,7 +173,7 @@ cudaError_t launch_march_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    return launch_chained(kern, grid, NT, M::BYTES, s, g, p, io, H);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<R>(grid, sms), s, g, p, io, H);
 }
 
 template <typename R, int TX, int TY, int NT, bool AUX, bool ISO>
@@ -184,6 +200,35 @@ __global__ void k_tsub2d(Geom g, Phys<R> p, const R* Tin, R* Tout)
     chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     march::tsub2d_site(g, p, Tin, Tout, x, y);
+}
+
+// S of them at once in FP32 (lf_tsub2d.cuh): one warp per strip and segment of H rows.
+template <int S, bool ISO>
+__global__ void __launch_bounds__(128) k_tsub2d_rows(Geom g, Phys<float> p, const float* Tin, float* Tout, int strips, int H)
+{
+    const int w = blockIdx.x * 4 + (threadIdx.x >> 5);
+    const int seg = w / strips, y0 = seg * H;
+    chain_wait();
+    if (y0 < g.ny)                               // for the whole warp
+        tsub::tsub2d_rows<S, ISO>(g, p, Tin, Tout, w - seg * strips, y0, min(y0 + H, g.ny));
+    chain_next();
+}
+
+template <int S>
+cudaError_t launch_tsub_rows(const Geom& g, const Phys<float>& p, const float* Tin, float* Tout, cudaStream_t s)
+{
+    int sms = 0;
+    const cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const int strips = ((g.nx + 3) / 4 + tsub::kQuads - 1) / tsub::kQuads;
+    // about sixteen warps per SM, segments of 4 to 64 rows (each reads 2 S rows more)
+    const int64_t want = (16 * (int64_t)sms + strips - 1) / strips;
+    int H = (int)((g.ny + want - 1) / want);
+    H = H < 4 ? 4 : (H > 64 ? 64 : H);
+    const int segs = (g.ny + H - 1) / H;
+    const dim3 grid((unsigned)(((int64_t)strips * segs + 3) / 4));
+    auto kern = g.stencil == LF_STENCIL_ISOTROPIC ? k_tsub2d_rows<S, true> : k_tsub2d_rows<S, false>;
+    return launch_chained(kern, grid, 128, 0, s, g, p, Tin, Tout, strips, H);
 }
 
 // The same sub-step with the isotropic 9-point Laplacian (lf_tile2d.cuh).
@@ -243,17 +288,35 @@ cudaError_t launch_step2d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, 
 }
 
 template <typename R>
-cudaError_t launch_tsub(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, cudaStream_t s)
+int tsub_fused(const Geom& g, int left)
+{
+    return sizeof(R) == 4 && g.d == 2 ? tsub::fused(left) : 1;
+}
+
+template <typename R>
+cudaError_t launch_tsub(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, int n, cudaStream_t s)
 {
     if (g.d == 3) return launch_tsub3d<R>(g, p, Tin, Tout, s);
-    dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8);
-    return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub2d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
-                                             : launch_chained(k_tsub2d<R>, grd, blk, 0, s, g, p, Tin, Tout);
+    if constexpr (sizeof(R) == 4) {
+        switch (n) {
+        case 1: return launch_tsub_rows<1>(g, p, Tin, Tout, s);
+        case 2: return launch_tsub_rows<2>(g, p, Tin, Tout, s);
+        case 3: return launch_tsub_rows<3>(g, p, Tin, Tout, s);
+        case 4: return launch_tsub_rows<4>(g, p, Tin, Tout, s);
+        default: return cudaErrorInvalidValue;
+        }
+    } else {
+        dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8);
+        return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub2d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
+                                                 : launch_chained(k_tsub2d<R>, grd, blk, 0, s, g, p, Tin, Tout);
+    }
 }
 
 template cudaError_t launch_step2d<float>(const Geom&, const Phys<float>&, const StepIO<float>&, bool, cudaStream_t);
 template cudaError_t launch_step2d<double>(const Geom&, const Phys<double>&, const StepIO<double>&, bool, cudaStream_t);
-template cudaError_t launch_tsub<float>(const Geom&, const Phys<float>&, const float*, float*, cudaStream_t);
-template cudaError_t launch_tsub<double>(const Geom&, const Phys<double>&, const double*, double*, cudaStream_t);
+template int tsub_fused<float>(const Geom&, int);
+template int tsub_fused<double>(const Geom&, int);
+template cudaError_t launch_tsub<float>(const Geom&, const Phys<float>&, const float*, float*, int, cudaStream_t);
+template cudaError_t launch_tsub<double>(const Geom&, const Phys<double>&, const double*, double*, int, cudaStream_t);
 
 }  // namespace lf
