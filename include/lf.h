@@ -251,7 +251,8 @@ int lf_load(lf_ctx* ctx, const char* path);
  *     lattice size), inputs prefetched with cp.async; (param >> 16) == 1
  *     selects CTAs of 64 threads (56 columns) instead of 128 (120 columns);
  *     with the isotropic stencils this one-lane march runs with sliding row
- *     sums;
+ *     sums; FP64 contexts with param 0 and up to 2^20 sites (isotropic: 2^19)
+ *     take one small tile per CTA instead;
  *   LF_VARIANT_TILE: one CTA per 2D tile, each stage of the step on the whole
  *     tile in shared memory (`param` ignored);
  *   LF_VARIANT_MARCH2 (default for 2D FP32; FP64 contexts run LF_VARIANT_MARCH

@@ -107,6 +107,9 @@ struct StepIO {
 template <typename R>
 cudaError_t launch_step2d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, bool aux,
                           cudaStream_t s);
+// the 2D step in FP64 on tiles (lf_step2d_f64.cu), and whether the lattice is small enough for it to be the default
+bool f64_tiles(const Geom& g);
+cudaError_t launch_step2d_f64(const Geom& g, const Phys<double>& p, const StepIO<double>& io, cudaStream_t s);
 template <typename R>
 cudaError_t launch_step3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, bool aux,
                           cudaStream_t s);

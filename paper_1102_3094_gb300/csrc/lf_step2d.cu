@@ -248,6 +248,9 @@ __global__ void k_tsub2d_iso(Geom g, Phys<R> p, const R* Tin, R* Tout)
 template <typename R>
 cudaError_t launch_step2d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, bool aux, cudaStream_t s)
 {
+    if constexpr (sizeof(R) == 8) {
+        if (!aux && g.variant == LF_VARIANT_MARCH && g.tune == 0 && f64_tiles(g)) return launch_step2d_f64(g, p, io, s);
+    }
     if (g.stencil == LF_STENCIL_ISOTROPIC) {           // the row marches or the tile kernel
         if constexpr (sizeof(R) == 4) {
             if (!aux && g.variant == LF_VARIANT_MARCH2 && g.ny >= 2) {
