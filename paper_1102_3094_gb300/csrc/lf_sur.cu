@@ -14,6 +14,7 @@
 
 #include "lf_ctx.cuh"
 #include "lf_sur.h"
+#include "lf_sur_conv.cuh"
 
 using namespace lf;
 
@@ -41,6 +42,7 @@ __global__ void k_norm_in(const float* __restrict__ raw, int B, int NY, int NX, 
                           __nv_bfloat16* __restrict__ x16, float* __restrict__ x4)
 {
     const int64_t N = (int64_t)B * NY * NX;
+    chain_next();                                // the first layer sets up meanwhile
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
         const int x = (int)(k % NX);
         const int64_t r = k / NX;
@@ -77,19 +79,6 @@ __global__ void k_norm_target(const float* __restrict__ raw, int B, int NY, int 
 #pragma unroll
         for (int c = 0; c < 4; ++c)
             t4[k * 4 + c] = (raw[(((int64_t)b * 4 + c) * NY + y) * NX + x] - (float)nm.offset[c]) * (float)(1.0 / nm.scale[c]);
-    }
-}
-
-__global__ void k_denorm(const float* __restrict__ y4, int B, int NY, int NX, lf_sur_norm nm, float* __restrict__ raw)
-{
-    const int64_t N = (int64_t)B * NY * NX;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(k % NX);
-        const int64_t r = k / NX;
-        const int y = (int)(r % NY), b = (int)(r / NY);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            raw[(((int64_t)b * 4 + c) * NY + y) * NX + x] = y4[k * 4 + c] * (float)nm.scale[c] + (float)nm.offset[c];
     }
 }
 
@@ -314,22 +303,60 @@ int refresh_bf16(lf_sur* s, int do_update, float lr)
     return cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
 }
 
-// keep_z: store each layer's pre-activation values for the backward pass
-// (training); a prediction does not need them
-int forward(lf_sur* s, const float* raw, int B, bool keep_z)
+sur::ConvArgs conv_args(const lf_sur* s, int B)
 {
-    const int NY = s->NY, NX = s->NX;
-    const int64_t N = (int64_t)B * NY * NX;
-    k_norm_in<<<blocks_for(N), 256, 0, s->stream>>>(raw, B, NY, NX, s->norm, s->x16, s->x4);
-    int rc = lf_sur_conv3x3(B, NY, NX, 16, 64, s->x16, s->wbf[0], s->b[0], 1, nullptr, nullptr, s->h[0], nullptr,
-                            keep_z ? s->z[0] : nullptr, nullptr, nullptr, s->err, s->stream);
-    for (int l = 1; l < 5 && rc == LF_OK; ++l)
-        rc = lf_sur_conv3x3(B, NY, NX, 64, 64, s->h[l - 1], s->wbf[l], s->b[l], 1, s->h[l - 1], nullptr, s->h[l],
-                            nullptr, keep_z ? s->z[l] : nullptr, nullptr, nullptr, s->err, s->stream);
-    if (rc == LF_OK)
-        rc = lf_sur_conv3x3(B, NY, NX, 64, 16, s->h[4], s->wbf[5], s->b[5], 0, nullptr, nullptr, nullptr, nullptr,
-                            nullptr, s->x4, s->y4, s->err, s->stream);
-    return rc;
+    sur::ConvArgs a{};
+    a.B = B;
+    a.NY = s->NY;
+    a.NX = s->NX;
+    a.err = s->err;
+    // the layers are launched so that each starts while the one before drains;
+    // the normalisation ahead of them is a plain launch, after whatever wrote
+    // the weights
+    a.old_weights = 1;
+    return a;
+}
+
+int run_conv(const lf_sur* s, int cin, int cout, const sur::ConvArgs& a)
+{
+    return sur::conv3x3(cin, cout, a, s->stream) == cudaSuccess ? LF_OK : LF_ECUDA;
+}
+
+// keep_z: store each layer's pre-activation values for the backward pass
+// (training); a prediction does not need them.  raw_out: the last layer writes
+// the prediction in raw units there instead of y4.
+int forward(lf_sur* s, const float* raw, int B, bool keep_z, float* raw_out)
+{
+    const int64_t N = (int64_t)B * s->NY * s->NX;
+    k_norm_in<<<blocks_for(N), 256, 0, s->stream>>>(raw, B, s->NY, s->NX, s->norm, s->x16, s->x4);
+    int rc = cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
+    for (int l = 0; l < 5 && rc == LF_OK; ++l) {
+        sur::ConvArgs a = conv_args(s, B);
+        a.in = l == 0 ? s->x16 : s->h[l - 1];
+        a.w = s->wbf[l];
+        a.bias = s->b[l];
+        a.relu = 1;
+        a.resid = l == 0 ? nullptr : s->h[l - 1];
+        a.out = s->h[l];
+        a.zout = keep_z ? s->z[l] : nullptr;
+        rc = run_conv(s, l == 0 ? 16 : 64, 64, a);
+    }
+    if (rc != LF_OK) return rc;
+    sur::ConvArgs a = conv_args(s, B);
+    a.in = s->h[4];
+    a.w = s->wbf[5];
+    a.bias = s->b[5];
+    a.x4 = s->x4;
+    if (raw_out) {
+        a.raw = raw_out;
+        for (int c = 0; c < 4; ++c) {
+            a.scale[c] = (float)s->norm.scale[c];
+            a.offset[c] = (float)s->norm.offset[c];
+        }
+    } else {
+        a.y4 = s->y4;
+    }
+    return run_conv(s, 64, 16, a);
 }
 
 // loss (host, FP64) and, when grads, every gradient into gw / gb
@@ -337,7 +364,7 @@ int loss_and_grads(lf_sur* s, const float* x, const float* y, int B, double* los
 {
     const int NY = s->NY, NX = s->NX;
     const int64_t N = (int64_t)B * NY * NX;
-    int rc = forward(s, x, B, grads);
+    int rc = forward(s, x, B, grads, nullptr);
     if (rc != LF_OK) return rc;
     k_norm_target<<<blocks_for(N), 256, 0, s->stream>>>(y, B, NY, NX, s->norm, s->t4);
     const unsigned mb = blocks_for(N);
@@ -539,10 +566,7 @@ int lf_sur_predict(lf_sur* s, const float* x, float* y, int B)
 {
     lf::NvtxRange nvtx_range("lf_sur_predict");
     if (!s || !x || !y || B < 1 || B > s->maxB) return LF_EINVAL;
-    int rc = forward(s, x, B, false);
-    if (rc != LF_OK) return rc;
-    k_denorm<<<blocks_for((int64_t)B * s->NY * s->NX), 256, 0, s->stream>>>(s->y4, B, s->NY, s->NX, s->norm, y);
-    return cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
+    return forward(s, x, B, false, y);
 }
 
 void lf_sur_destroy(lf_sur* s)

@@ -39,26 +39,11 @@
 
 #include "lf_internal.cuh"
 #include "lf_sur.h"
+#include "lf_sur_conv.cuh"
 #include "lf_tc.cuh"
 
 namespace lf {
 namespace sur {
-
-struct ConvArgs {
-    const __nv_bfloat16* in;     // padded NHWC, CIN channels
-    const __nv_bfloat16* w;      // [9][COUT][CIN], tap t = 3 (dy + 1) + (dx + 1)
-    const float* bias;           // [COUT] or null
-    const __nv_bfloat16* resid;  // padded NHWC COUT, added after the activation, or null
-    const __nv_bfloat16* mask;   // padded NHWC COUT: out2 = out * (mask > 0), or null
-    __nv_bfloat16* out;          // padded NHWC COUT, or null
-    __nv_bfloat16* out2;         // padded NHWC COUT (masked copy of out), or null
-    __nv_bfloat16* zout;         // padded NHWC COUT: pre-activation value, or null
-    const float* x4;             // [B][NY][NX][4]: y4 = x4 + (acc + bias)[0..3], or null
-    float* y4;
-    int relu;
-    int B, NY, NX;
-    int* err;
-};
 
 template <int CIN, int COUT>
 struct ConvSmem {
@@ -168,6 +153,11 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
     const bool start = *abort_flag == 0;
+    // A convolution of one lattice takes about 10 us, of which launch, setup and
+    // weights were 5: the successor may come in now (not before this CTA has its
+    // tensor memory, which the successor's would otherwise take from it).
+    chain_next();
+    if (!a.old_weights || warp != EW) chain_wait();
 
     if (warp == EW) {
         // TMA producer: the weights, then padded rows ya .. yb + 1 of each
@@ -179,6 +169,7 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
                 for (int t = 0; t < 9; ++t)
                     tc::tma_load_3d(sB + (3 * (t % 3) + t / 3) * S::B_TAP, &tw, 0, 0, t, wbar);
             }
+            if (a.old_weights) chain_wait();
             uint32_t ld = 0;
             bool ok = true;
             for (int64_t q = r0; q < r1 && ok;) {
@@ -363,6 +354,12 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
 #pragma unroll
                     for (int i = 0; i < 4; ++i) a.y4[q4 + i] = a.x4[q4 + i] + v[i];
                 }
+                if (a.raw && c0 == 0) {
+                    const int64_t q4 = (((int64_t)g.b * NY + y) * NX + x) * 4, np = (int64_t)NY * NX;
+                    float* d = a.raw + ((int64_t)g.b * 4 * NY + y) * NX + x;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) d[i * np] = fmaf(a.x4[q4 + i] + v[i], a.scale[i], a.offset[i]);
+                }
                 __align__(16) __nv_bfloat16 hz[16], ho[16], hm[16];
                 if (a.zout)
 #pragma unroll
@@ -465,8 +462,7 @@ cudaError_t launch_conv(const ConvArgs& a, cudaStream_t s)
     if (cudaError_t e = device_sms(&sms); e != cudaSuccess) return e;
     const int64_t rows = (int64_t)a.B * (a.NX / 128) * a.NY;
     const int blocks = (int)(rows < sms ? rows : sms);
-    k_conv3x3<CIN, COUT><<<blocks, conv_threads<COUT>(), S::BYTES, s>>>(m, mw, a);
-    return cudaGetLastError();
+    return launch_chained(k_conv3x3<CIN, COUT>, blocks, conv_threads<COUT>(), S::BYTES, s, m, mw, a);
 }
 
 cudaError_t conv3x3(int cin, int cout, const ConvArgs& a, cudaStream_t s)
