@@ -344,6 +344,10 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
                         rp[0] = *reinterpret_cast<const uint4*>(row + (c0 / 8) * S::LBO_A + px * 16);
                         rp[1] = *reinterpret_cast<const uint4*>(row + (c0 / 8 + 1) * S::LBO_A + px * 16);
                     }
+                    // the slot is refilled by TMA, another proxy: without this fence a row
+                    // arriving early was read in place of the residual (rows where the
+                    // epilogue is behind the MMAs)
+                    tc::fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(&empty[sl]);
                 }
