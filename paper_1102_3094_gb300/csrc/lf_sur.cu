@@ -36,85 +36,119 @@ uint64_t splitmix(uint64_t& s)
 
 // ---- small kernels ----------------------------------------------------------
 
+// What a training step accumulates with atomics: the bias gradients and the
+// squared norm of all gradients (null outside of training).
+struct GradSums {
+    float* db[kLayers];
+    double* norm2;
+};
+
 // raw fields [B][4][NY][NX] (phi, T, ux, uy) -> x16 padded NHWC BF16 (channels
 // 4..15 zero, halo per the lattice) and x4 = normalised FP32 [B][NY][NX][4]
-__global__ void k_norm_in(const float* __restrict__ raw, int B, int NY, int NX, lf_sur_norm nm,
-                          __nv_bfloat16* __restrict__ x16, float* __restrict__ x4)
+__global__ void __launch_bounds__(256) k_norm_in(const float* __restrict__ raw, int B, int NY, int NX, lf_sur_norm nm,
+                                                 __nv_bfloat16* __restrict__ x16, float4* __restrict__ x4,
+                                                 GradSums zero)
 {
-    const int64_t N = (int64_t)B * NY * NX;
+    if (blockIdx.x == 0 && zero.norm2) {         // the sums of the training step that begins here
+        for (int l = 0; l < kLayers; ++l)
+            if (threadIdx.x < (l == kLayers - 1 ? 16u : 64u)) zero.db[l][threadIdx.x] = 0.f;
+        if (threadIdx.x == 0) *zero.norm2 = 0.0;
+    }
+    const int rows = B * NY;
+    float is[4], of[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        is[c] = (float)(1.0 / nm.scale[c]);
+        of[c] = (float)nm.offset[c];
+    }
+    const int64_t np = (int64_t)NY * NX;
     chain_next();                                // the first layer sets up meanwhile
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(k % NX);
-        const int64_t r = k / NX;
-        const int y = (int)(r % NY), b = (int)(r / NY);
-        __align__(16) __nv_bfloat16 v[16];
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+        const int b = r / NY, y = r - b * NY;
+        const float* f = raw + b * 4 * np + (int64_t)y * NX;
+        __nv_bfloat16* xr = x16 + (((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + 1) * 16;
+        for (int x = threadIdx.x; x < NX; x += 256) {
+            float s[4];
+            uint32_t v[4];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float s = (raw[(((int64_t)b * 4 + c) * NY + y) * NX + x] - (float)nm.offset[c]) * (float)(1.0 / nm.scale[c]);
-            x4[k * 4 + c] = s;
-            v[c] = __float2bfloat16_rn(s);
-        }
-        const int64_t po = ((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + x + 1;
-        uint4* d = reinterpret_cast<uint4*>(x16 + po * 16);
-        d[0] = reinterpret_cast<uint4*>(v)[0];
-        d[1] = reinterpret_cast<uint4*>(v)[1];
-        if (x == 0 || x == NX - 1) {
-            const int64_t ph = ((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + (x == 0 ? NX + 1 : 0);
-            uint4* dh = reinterpret_cast<uint4*>(x16 + ph * 16);
-            dh[0] = reinterpret_cast<uint4*>(v)[0];
-            dh[1] = reinterpret_cast<uint4*>(v)[1];
+            for (int c = 0; c < 4; ++c) {
+                s[c] = (f[c * np + x] - of[c]) * is[c];
+                v[c] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(s[c]));
+            }
+            x4[(int64_t)r * NX + x] = make_float4(s[0], s[1], s[2], s[3]);
+            const uint4 w0 = make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, 0, 0), z = make_uint4(0, 0, 0, 0);
+            uint4* d = reinterpret_cast<uint4*>(xr + (int64_t)x * 16);
+            d[0] = w0;
+            d[1] = z;
+            if (x == 0 || x == NX - 1) {         // the periodic halo column
+                uint4* dh = reinterpret_cast<uint4*>(xr + (int64_t)(x == 0 ? NX : -1) * 16);
+                dh[0] = w0;
+                dh[1] = z;
+            }
         }
     }
 }
 
-__global__ void k_norm_target(const float* __restrict__ raw, int B, int NY, int NX, lf_sur_norm nm, float* __restrict__ t4)
-{
-    const int64_t N = (int64_t)B * NY * NX;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(k % NX);
-        const int64_t r = k / NX;
-        const int y = (int)(r % NY), b = (int)(r / NY);
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-            t4[k * 4 + c] = (raw[(((int64_t)b * 4 + c) * NY + y) * NX + x] - (float)nm.offset[c]) * (float)(1.0 / nm.scale[c]);
-    }
-}
-
-// MSE over B NY NX 4 outputs: per-block FP64 partial of sum (y - t)^2, and the
-// gradient g = 2 (y - t) / count into the padded 16-channel BF16 tensor
-__global__ void k_mse(const float* __restrict__ y4, const float* __restrict__ t4, int B, int NY, int NX,
-                      double* __restrict__ part, __nv_bfloat16* __restrict__ g16)
+// MSE over B NY NX 4 outputs against the raw target fields [B][4][NY][NX]
+// (normalised here): per-block FP64 partial of sum (y - t)^2; with gradients,
+// g = 2 (y - t) / count into the padded 16-channel BF16 tensor and its channel
+// sums, the last layer's bias gradient, into db[0 .. 3].
+__global__ void __launch_bounds__(256) k_mse(const float4* __restrict__ y4, const float* __restrict__ raw, int B, int NY,
+                                             int NX, lf_sur_norm nm, double* __restrict__ part,
+                                             __nv_bfloat16* __restrict__ g16, float* __restrict__ db)
 {
     __shared__ double red[256];
-    const int64_t N = (int64_t)B * NY * NX;
-    const float inv = (float)(2.0 / (4.0 * (double)N));
-    double acc = 0.0;
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(k % NX);
-        const int64_t r = k / NX;
-        const int y = (int)(r % NY), b = (int)(r / NY);
-        __align__(16) __nv_bfloat16 v[16];
+    const int rows = B * NY;
+    const float inv = (float)(2.0 / (4.0 * (double)rows * NX));
+    float is[4], of[4], bs[4] = {};
 #pragma unroll
-        for (int c = 0; c < 16; ++c) v[c] = __float2bfloat16_rn(0.f);
+    for (int c = 0; c < 4; ++c) {
+        is[c] = (float)(1.0 / nm.scale[c]);
+        of[c] = (float)nm.offset[c];
+    }
+    double acc = 0.0;
+    const int64_t np = (int64_t)NY * NX;
+    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+        const int b = r / NY, y = r - b * NY;
+        const float* t = raw + b * 4 * np + (int64_t)y * NX;
+        const int64_t row = (((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + 1) * 16;
+        for (int x = threadIdx.x; x < NX; x += 256) {
+            const float4 q = y4[(int64_t)r * NX + x];
+            const float yv[4] = {q.x, q.y, q.z, q.w};
+            uint32_t v[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float d = yv[c] - __fmul_rn(t[c * np + x] - of[c], is[c]);
+                acc += (double)d * d;
+                const __nv_bfloat16 h = __float2bfloat16_rn(inv * d);
+                v[c] = (uint32_t)__bfloat16_as_ushort(h);
+                bs[c] += __bfloat162float(h);
+            }
+            if (g16) {
+                const uint4 w0 = make_uint4(v[0] | v[1] << 16, v[2] | v[3] << 16, 0, 0), z = make_uint4(0, 0, 0, 0);
+                uint4* d = reinterpret_cast<uint4*>(g16 + row + (int64_t)x * 16);
+                d[0] = w0;
+                d[1] = z;
+                if (x == 0 || x == NX - 1) {     // the periodic halo column
+                    uint4* dh = reinterpret_cast<uint4*>(g16 + row + (int64_t)(x == 0 ? NX : -1) * 16);
+                    dh[0] = w0;
+                    dh[1] = z;
+                }
+            }
+        }
+    }
+    if (g16) {
+        __shared__ float rb[8][4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            const float d = y4[k * 4 + c] - t4[k * 4 + c];
-            acc += (double)d * d;
-            v[c] = __float2bfloat16_rn(inv * d);
+            for (int o = 16; o > 0; o >>= 1) bs[c] += __shfl_xor_sync(0xffffffffu, bs[c], o);
+            if ((threadIdx.x & 31) == 0) rb[threadIdx.x >> 5][c] = bs[c];
         }
-        if (g16) {
-            const int64_t po = ((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + x + 1;
-            uint4* dd = reinterpret_cast<uint4*>(g16 + po * 16);
-            dd[0] = reinterpret_cast<uint4*>(v)[0];
-            dd[1] = reinterpret_cast<uint4*>(v)[1];
-            if (x == 0 || x == NX - 1) {
-                const int64_t ph = ((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + (x == 0 ? NX + 1 : 0);
-                uint4* dh = reinterpret_cast<uint4*>(g16 + ph * 16);
-                dh[0] = reinterpret_cast<uint4*>(v)[0];
-                dh[1] = reinterpret_cast<uint4*>(v)[1];
-            }
+        __syncthreads();
+        if (threadIdx.x < 4) {
+            float t = 0.f;
+            for (int w = 0; w < 8; ++w) t += rb[w][threadIdx.x];
+            atomicAdd(&db[threadIdx.x], t);
         }
     }
     red[threadIdx.x] = acc;
@@ -126,58 +160,6 @@ __global__ void k_mse(const float* __restrict__ y4, const float* __restrict__ t4
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-// Bias gradient: db[o] = sum over interior pixels of g[p][o] (FP32 block sums,
-// atomics).  Bound by reading g once (134 MB at 16 x 256^2 and 64 channels).  A
-// block takes whole lattice rows, which are contiguous in the padded layout, so
-// no pixel index is divided; a thread reads 8 channels of a pixel with one
-// 16-byte load, four loads in flight, and keeps their sums.  (One 2-byte load
-// and two 64-bit divisions per value took 483 us there; this takes 27 us.)
-template <int C>
-__global__ void __launch_bounds__(256) k_bias_grad(const __nv_bfloat16* __restrict__ g, int B, int NY, int NX,
-                                                   float* __restrict__ db)
-{
-    constexpr int TP = C / 8;                    // threads per pixel
-    constexpr int PX = 256 / TP;                 // pixels per block and pass
-    __shared__ float red[PX][C];
-    const int cg = threadIdx.x % TP, sub = threadIdx.x / TP;
-    float acc[8] = {};
-    const int rows = B * NY;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int b = r / NY, y = r - b * NY;
-        const uint4* row = reinterpret_cast<const uint4*>(g + (((int64_t)b * (NY + 2) + y + 1) * (NX + 2) + 1) * C) + cg;
-        for (int x = sub; x < NX; x += 4 * PX) {
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = x + u * PX < NX ? row[(x + u * PX) * TP] : make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {    // a BF16 is the upper half of an FP32
-                    acc[2 * i] += __uint_as_float(w[i] << 16);
-                    acc[2 * i + 1] += __uint_as_float(w[i] & 0xFFFF0000u);
-                }
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 8; ++i) red[sub][cg * 8 + i] = acc[i];
-    __syncthreads();
-    for (int n = PX / 2; n > 0; n >>= 1) {
-        for (int k = threadIdx.x; k < n * C; k += 256) red[k / C][k % C] += red[k / C + n][k % C];
-        __syncthreads();
-    }
-    if (threadIdx.x < C) atomicAdd(&db[threadIdx.x], red[0][threadIdx.x]);
-}
-
-cudaError_t bias_grad(const __nv_bfloat16* g, int C, int B, int NY, int NX, float* db, cudaStream_t s)
-{
-    const int rows = B * NY, blocks = std::min(rows, 152 * 4);
-    if (C == 64) k_bias_grad<64><<<blocks, 256, 0, s>>>(g, B, NY, NX, db);
-    else k_bias_grad<16><<<blocks, 256, 0, s>>>(g, B, NY, NX, db);
-    return cudaGetLastError();
-}
-
 // Adam on FP32 master parameters; writes the BF16 weights for the forward pass
 // and the tap-flipped, transposed BF16 copies for the backward data pass.
 struct AdamLayer {
@@ -187,29 +169,36 @@ struct AdamLayer {
     int cin, cout;
 };
 
-// Squared norm of one layer's gradients (weights and biases) added to *acc.
-__global__ void k_grad_sumsq(const float* __restrict__ gw, int nw, const float* __restrict__ gb, int nb, double* acc)
+struct AdamLayers {
+    AdamLayer l[kLayers];
+};
+
+// Squared norm of all gradients (one block of n floats) added to *acc.
+__global__ void k_grad_sumsq(const float* __restrict__ g, int n, double* acc)
 {
     double v = 0.0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nw + nb; k += gridDim.x * blockDim.x) {
-        const double g = k < nw ? gw[k] : gb[k - nw];
-        v += g * g;
-    }
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) v += (double)g[k] * g[k];
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) atomicAdd(acc, v);
 }
 
 // Adam with the gradients scaled by min(1, clip / ||g||) (global norm
-// clipping; clip = 0 leaves them as they are).
-__global__ void k_adam(AdamLayer L, float lr, float b1, float b2, float eps, float c1, float c2, int do_update,
+// clipping; clip = 0 leaves them as they are); blockIdx.y is the layer.
+__global__ void k_adam(AdamLayers layers, float lr, float b1, float b2, float eps, float c1, float c2, int do_update,
                        const double* gnorm2, float clip)
 {
+    const AdamLayer& L = layers.l[blockIdx.y];
     const int nw = 9 * L.cout * L.cin;
-    float gs = 1.f;
-    if (do_update && clip > 0.f) {
-        const double n = sqrt(*gnorm2);
-        if (n > (double)clip) gs = (float)((double)clip / n);
+    __shared__ float scale;                      // one FP64 root and quotient per block, not per thread
+    if (threadIdx.x == 0) {
+        scale = 1.f;
+        if (do_update && clip > 0.f) {
+            const double n = sqrt(*gnorm2);
+            if (n > (double)clip) scale = (float)((double)clip / n);
+        }
     }
+    __syncthreads();
+    const float gs = scale;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < nw + L.cout; k += gridDim.x * blockDim.x) {
         if (k < nw) {
             float w = L.w[k];
@@ -251,18 +240,19 @@ struct lf_sur {
     cudaStream_t stream;
     unsigned char* block;        // one device allocation for everything below
     size_t bytes;
-    // parameters (FP32 master), Adam moments, gradients; BF16 copies
+    // parameters (FP32 master), Adam moments, gradients: one block each, layer by
+    // layer (weights, bias) as lf_sur_param_count has them; BF16 copies
     float* w[kLayers]; float* m[kLayers]; float* v[kLayers]; float* gw[kLayers];
     float* b[kLayers]; float* mb[kLayers]; float* vb[kLayers]; float* gb[kLayers];
     __nv_bfloat16* wbf[kLayers]; __nv_bfloat16* wtbf[kLayers];
     // activations (padded NHWC BF16)
     __nv_bfloat16* x16;          // input
     __nv_bfloat16* h[kLayers - 1];   // h1 .. h5 (64 ch)
-    __nv_bfloat16* z[kLayers - 1];   // z1 .. z5 (pre-activations, masks)
+    uint16_t* zb[kLayers - 1];   // (z1 > 0) .. (z5 > 0): pre-activation signs, one bit each
     __nv_bfloat16* g16;          // dL/dz6 (16 ch)
     __nv_bfloat16* ga; __nv_bfloat16* gb2; __nv_bfloat16* gz;   // dL/dh ping-pong and dL/dz (64 ch)
     __nv_bfloat16* gz_alt;
-    float* x4; float* y4; float* t4;
+    float* x4; float* y4;
     float* part;                 // weight-gradient partials
     size_t part_floats;
     double* loss_part;           // k_mse block partials
@@ -289,17 +279,14 @@ int refresh_bf16(lf_sur* s, int do_update, float lr)
     const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
     const float c1 = do_update ? (float)(1.0 / (1.0 - std::pow(b1, s->step))) : 1.f;
     const float c2 = do_update ? (float)(1.0 / (1.0 - std::pow(b2, s->step))) : 1.f;
-    if (do_update) {
-        if (cudaMemsetAsync(s->gnorm2, 0, sizeof(double), s->stream) != cudaSuccess) return LF_ECUDA;
-        for (int l = 0; l < kLayers; ++l)
-            k_grad_sumsq<<<64, 256, 0, s->stream>>>(s->gw[l], (int)wcount(l), s->gb[l], kCout[l], s->gnorm2);
-    }
-    for (int l = 0; l < kLayers; ++l) {
-        AdamLayer L{s->w[l], s->m[l], s->v[l], s->gw[l], s->b[l], s->mb[l], s->vb[l], s->gb[l], s->wbf[l], s->wtbf[l],
-                    kCin[l], kCout[l]};
-        k_adam<<<blocks_for((int64_t)wcount(l) + kCout[l]), 256, 0, s->stream>>>(L, lr, b1, b2, eps, c1, c2, do_update,
-                                                                               s->gnorm2, s->clip);
-    }
+    const int np = (int)lf_sur_param_count();
+    if (do_update) k_grad_sumsq<<<152, 256, 0, s->stream>>>(s->gw[0], np, s->gnorm2);
+    AdamLayers L;
+    for (int l = 0; l < kLayers; ++l)
+        L.l[l] = AdamLayer{s->w[l], s->m[l], s->v[l], s->gw[l], s->b[l], s->mb[l], s->vb[l], s->gb[l], s->wbf[l], s->wtbf[l],
+                           kCin[l], kCout[l]};
+    const dim3 grid(blocks_for((int64_t)wcount(1) + kCout[1]), kLayers);
+    k_adam<<<grid, 256, 0, s->stream>>>(L, lr, b1, b2, eps, c1, c2, do_update, s->gnorm2, s->clip);
     return cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
 }
 
@@ -322,13 +309,18 @@ int run_conv(const lf_sur* s, int cin, int cout, const sur::ConvArgs& a)
     return sur::conv3x3(cin, cout, a, s->stream) == cudaSuccess ? LF_OK : LF_ECUDA;
 }
 
-// keep_z: store each layer's pre-activation values for the backward pass
+// keep_z: store the signs of each layer's pre-activations for the backward pass
 // (training); a prediction does not need them.  raw_out: the last layer writes
 // the prediction in raw units there instead of y4.
 int forward(lf_sur* s, const float* raw, int B, bool keep_z, float* raw_out)
 {
-    const int64_t N = (int64_t)B * s->NY * s->NX;
-    k_norm_in<<<blocks_for(N), 256, 0, s->stream>>>(raw, B, s->NY, s->NX, s->norm, s->x16, s->x4);
+    GradSums zero{};
+    if (keep_z) {                                // a training step begins
+        for (int l = 0; l < kLayers; ++l) zero.db[l] = s->gb[l];
+        zero.norm2 = s->gnorm2;
+    }
+    k_norm_in<<<(unsigned)std::min(B * s->NY, 152 * 8), 256, 0, s->stream>>>(raw, B, s->NY, s->NX, s->norm, s->x16,
+                                                                             (float4*)s->x4, zero);
     int rc = cudaGetLastError() == cudaSuccess ? LF_OK : LF_ECUDA;
     for (int l = 0; l < 5 && rc == LF_OK; ++l) {
         sur::ConvArgs a = conv_args(s, B);
@@ -338,7 +330,7 @@ int forward(lf_sur* s, const float* raw, int B, bool keep_z, float* raw_out)
         a.relu = 1;
         a.resid = l == 0 ? nullptr : s->h[l - 1];
         a.out = s->h[l];
-        a.zout = keep_z ? s->z[l] : nullptr;
+        a.zbits = keep_z ? s->zb[l] : nullptr;
         rc = run_conv(s, l == 0 ? 16 : 64, 64, a);
     }
     if (rc != LF_OK) return rc;
@@ -366,31 +358,39 @@ int loss_and_grads(lf_sur* s, const float* x, const float* y, int B, double* los
     const int64_t N = (int64_t)B * NY * NX;
     int rc = forward(s, x, B, grads, nullptr);
     if (rc != LF_OK) return rc;
-    k_norm_target<<<blocks_for(N), 256, 0, s->stream>>>(y, B, NY, NX, s->norm, s->t4);
-    const unsigned mb = blocks_for(N);
-    k_mse<<<mb, 256, 0, s->stream>>>(s->y4, s->t4, B, NY, NX, s->loss_part, grads ? s->g16 : nullptr);
+    const unsigned mb = (unsigned)std::min(B * NY, 152 * 4);
+    k_mse<<<mb, 256, 0, s->stream>>>((const float4*)s->y4, y, B, NY, NX, s->norm, s->loss_part, grads ? s->g16 : nullptr,
+                                     s->gb[kLayers - 1]);
+    if (cudaGetLastError() != cudaSuccess) return LF_ECUDA;
     if (grads) {
-        for (int l = 0; l < kLayers; ++l) cudaMemsetAsync(s->gb[l], 0, sizeof(float) * kCout[l], s->stream);
         // layer 6: dW6 from h5 and g16; dL/dh5 = conv(g16, W6'), mask by z5 -> dL/dz5
         const __nv_bfloat16* hin[kLayers] = {s->x16, s->h[0], s->h[1], s->h[2], s->h[3], s->h[4]};
+        // every convolution leaves the sums of the dL/dz it writes: that layer's bias gradient
+        auto data_grad = [&](int cin, const __nv_bfloat16* g, int l, const __nv_bfloat16* gh, __nv_bfloat16* gh_next,
+                             __nv_bfloat16* gz_next) {
+            sur::ConvArgs a = conv_args(s, B);
+            a.in = g;
+            a.w = s->wtbf[l];
+            a.resid = gh;
+            a.mbits = s->zb[l - 1];
+            a.out = gh_next;
+            a.out2 = gz_next;
+            a.bsum = s->gb[l - 1];
+            return run_conv(s, cin, 64, a);
+        };
         rc = lf_sur_conv3x3_wgrad(B, NY, NX, 64, 16, s->h[4], s->g16, s->part, s->part_floats, s->gw[5], s->err,
                                   s->stream);
-        bias_grad(s->g16, 16, B, NY, NX, s->gb[5], s->stream);
         __nv_bfloat16* gh = s->ga;       // dL/dh_l
         __nv_bfloat16* gz = s->gz;       // dL/dz_l
-        if (rc == LF_OK)
-            rc = lf_sur_conv3x3(B, NY, NX, 16, 64, s->g16, s->wtbf[5], nullptr, 0, nullptr, s->z[4], gh, gz, nullptr,
-                                nullptr, nullptr, s->err, s->stream);
+        if (rc == LF_OK) rc = data_grad(16, s->g16, 5, nullptr, gh, gz);
         // layers 5 .. 2: dW_l from h_{l-1} and dL/dz_l; dL/dh_{l-1} = dL/dh_l + conv(dL/dz_l, W_l')
+        // (of layer 1 only dL/dz_1 is needed)
         for (int l = 4; l >= 1 && rc == LF_OK; --l) {
             rc = lf_sur_conv3x3_wgrad(B, NY, NX, 64, 64, hin[l], gz, s->part, s->part_floats, s->gw[l], s->err,
                                       s->stream);
-            bias_grad(gz, 64, B, NY, NX, s->gb[l], s->stream);
             __nv_bfloat16* gh_next = (gh == s->ga) ? s->gb2 : s->ga;
             __nv_bfloat16* gz_next = (gz == s->gz) ? s->gz_alt : s->gz;
-            if (rc == LF_OK)
-                rc = lf_sur_conv3x3(B, NY, NX, 64, 64, gz, s->wtbf[l], nullptr, 0, gh, s->z[l - 1], gh_next, gz_next,
-                                    nullptr, nullptr, nullptr, s->err, s->stream);
+            if (rc == LF_OK) rc = data_grad(64, gz, l, gh, l > 1 ? gh_next : nullptr, gz_next);
             gh = gh_next;
             gz = gz_next;
         }
@@ -398,7 +398,6 @@ int loss_and_grads(lf_sur* s, const float* x, const float* y, int B, double* los
         if (rc == LF_OK)
             rc = lf_sur_conv3x3_wgrad(B, NY, NX, 16, 64, s->x16, gz, s->part, s->part_floats, s->gw[0], s->err,
                                       s->stream);
-        bias_grad(gz, 64, B, NY, NX, s->gb[0], s->stream);
     }
     if (rc != LF_OK) return rc;
     std::vector<double> lp(mb);
@@ -432,9 +431,10 @@ int lf_sur_create(int NY, int NX, int max_batch, uint64_t seed, const lf_sur_nor
                                lf_sur_wgrad_scratch_floats(64, 16)});
     size_t bytes = 0;
     for (int l = 0; l < kLayers; ++l)
-        bytes += 4 * a256(4 * wcount(l)) + 4 * a256(4 * (size_t)kCout[l]) + 2 * a256(2 * wcount(l));
-    bytes += a256(2 * pad_px * 16) * 2 + a256(2 * pad_px * 64) * (2 * 5 + 4);
-    bytes += 3 * a256(4 * px * 4) + a256(4 * s->part_floats) + a256(8 * 152 * 8) + 256 + 256;
+        bytes += 2 * a256(2 * wcount(l));
+    bytes += 4 * a256(4 * lf_sur_param_count());
+    bytes += a256(2 * pad_px * 16) * 2 + a256(2 * pad_px * 64) * (5 + 4) + a256(8 * px) * 5;
+    bytes += 2 * a256(4 * px * 4) + a256(4 * s->part_floats) + a256(8 * 152 * 8) + 256 + 256;
     if (cudaMalloc((void**)&s->block, bytes) != cudaSuccess) {
         cudaGetLastError();
         delete s;
@@ -443,22 +443,28 @@ int lf_sur_create(int NY, int NX, int max_batch, uint64_t seed, const lf_sur_nor
     s->bytes = bytes;
     unsigned char* p = s->block;
     auto take = [&](size_t n) { unsigned char* r = p; p += a256(n); return r; };
+    // every layer's weights and bias are multiples of 16 floats, so all of these start on 64 bytes
+    float* pw = (float*)take(4 * lf_sur_param_count());
+    float* pm = (float*)take(4 * lf_sur_param_count());
+    float* pv = (float*)take(4 * lf_sur_param_count());
+    float* pg = (float*)take(4 * lf_sur_param_count());
     for (int l = 0; l < kLayers; ++l) {
-        s->w[l] = (float*)take(4 * wcount(l)); s->m[l] = (float*)take(4 * wcount(l));
-        s->v[l] = (float*)take(4 * wcount(l)); s->gw[l] = (float*)take(4 * wcount(l));
-        s->b[l] = (float*)take(4 * kCout[l]); s->mb[l] = (float*)take(4 * kCout[l]);
-        s->vb[l] = (float*)take(4 * kCout[l]); s->gb[l] = (float*)take(4 * kCout[l]);
+        const size_t nw = wcount(l), nl = nw + kCout[l];
+        s->w[l] = pw; s->b[l] = pw + nw; pw += nl;
+        s->m[l] = pm; s->mb[l] = pm + nw; pm += nl;
+        s->v[l] = pv; s->vb[l] = pv + nw; pv += nl;
+        s->gw[l] = pg; s->gb[l] = pg + nw; pg += nl;
         s->wbf[l] = (__nv_bfloat16*)take(2 * wcount(l)); s->wtbf[l] = (__nv_bfloat16*)take(2 * wcount(l));
     }
     s->x16 = (__nv_bfloat16*)take(2 * pad_px * 16);
     s->g16 = (__nv_bfloat16*)take(2 * pad_px * 16);
     for (int l = 0; l < 5; ++l) s->h[l] = (__nv_bfloat16*)take(2 * pad_px * 64);
-    for (int l = 0; l < 5; ++l) s->z[l] = (__nv_bfloat16*)take(2 * pad_px * 64);
+    for (int l = 0; l < 5; ++l) s->zb[l] = (uint16_t*)take(8 * px);
     s->ga = (__nv_bfloat16*)take(2 * pad_px * 64);
     s->gb2 = (__nv_bfloat16*)take(2 * pad_px * 64);
     s->gz = (__nv_bfloat16*)take(2 * pad_px * 64);
     s->gz_alt = (__nv_bfloat16*)take(2 * pad_px * 64);
-    s->x4 = (float*)take(4 * px * 4); s->y4 = (float*)take(4 * px * 4); s->t4 = (float*)take(4 * px * 4);
+    s->x4 = (float*)take(4 * px * 4); s->y4 = (float*)take(4 * px * 4);
     s->part = (float*)take(4 * s->part_floats);
     s->loss_part = (double*)take(8 * 152 * 8);
     s->err = (int*)take(4);
@@ -508,30 +514,16 @@ size_t lf_sur_param_count(void)
 int lf_sur_get_params(lf_sur* s, float* host)
 {
     if (!s || !host) return LF_EINVAL;
-    size_t off = 0;
-    for (int l = 0; l < kLayers; ++l) {
-        if (cudaMemcpyAsync(host + off, s->w[l], 4 * wcount(l), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += wcount(l);
-        if (cudaMemcpyAsync(host + off, s->b[l], 4 * kCout[l], cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += kCout[l];
-    }
+    if (cudaMemcpyAsync(host, s->w[0], 4 * lf_sur_param_count(), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+        return LF_ECUDA;
     return wait_stream(s->stream);
 }
 
 int lf_sur_set_params(lf_sur* s, const float* host)
 {
     if (!s || !host) return LF_EINVAL;
-    size_t off = 0;
-    for (int l = 0; l < kLayers; ++l) {
-        if (cudaMemcpyAsync(s->w[l], host + off, 4 * wcount(l), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += wcount(l);
-        if (cudaMemcpyAsync(s->b[l], host + off, 4 * kCout[l], cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += kCout[l];
-    }
+    if (cudaMemcpyAsync(s->w[0], host, 4 * lf_sur_param_count(), cudaMemcpyHostToDevice, s->stream) != cudaSuccess)
+        return LF_ECUDA;
     int rc = refresh_bf16(s, 0, 0.f);
     return rc == LF_OK ? sync_check(s) : rc;
 }
@@ -541,15 +533,8 @@ int lf_sur_grads(lf_sur* s, const float* x, const float* y, int B, double* loss,
     if (!s || !x || !y || !loss || B < 1 || B > s->maxB) return LF_EINVAL;
     int rc = loss_and_grads(s, x, y, B, loss, grads_host != nullptr);
     if (rc != LF_OK || !grads_host) return rc;
-    size_t off = 0;
-    for (int l = 0; l < kLayers; ++l) {
-        if (cudaMemcpyAsync(grads_host + off, s->gw[l], 4 * wcount(l), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += wcount(l);
-        if (cudaMemcpyAsync(grads_host + off, s->gb[l], 4 * kCout[l], cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
-            return LF_ECUDA;
-        off += kCout[l];
-    }
+    if (cudaMemcpyAsync(grads_host, s->gw[0], 4 * lf_sur_param_count(), cudaMemcpyDeviceToHost, s->stream) != cudaSuccess)
+        return LF_ECUDA;
     return sync_check(s);
 }
 

@@ -22,6 +22,12 @@ struct ConvArgs {
     float* y4;
     float* raw;                  // [B][4][NY][NX]: y4 scale + offset in place of y4, or null
     float scale[4], offset[4];
+    // training: one bit per pre-activation value, (value > 0), [B NY][4][NX]
+    // 16-channel words of COUT = 64: written by the forward pass in place of
+    // zout, read by the backward pass in place of mask
+    uint16_t* zbits;
+    const uint16_t* mbits;
+    float* bsum;                 // [COUT] += sums over pixels of out2 (the next bias gradient), or null
     int relu;
     int B, NY, NX;
     int* err;
@@ -31,6 +37,7 @@ struct ConvArgs {
     int old_weights;
 };
 
+// `mbits` selects the backward form: acc (+ resid) -> out (may be null) and out2 = out where the bit is set.
 cudaError_t conv3x3(int cin, int cout, const ConvArgs& a, cudaStream_t s);
 
 }  // namespace sur
