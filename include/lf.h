@@ -260,7 +260,8 @@ int lf_load(lf_ctx* ctx, const char* path);
  *     march away from their common row, carried in the two lanes of packed
  *     FP32x2 arithmetic; (param & 0xFFFF) = rows per segment (0 = chosen from
  *     the lattice size and the SM count), (param >> 16) == 1 selects CTAs of
- *     64 threads (56 columns) instead of 128 (120 columns); with the
+ *     64 threads (56 columns) instead of 128 (120 columns; param 0 chooses the
+ *     width too); with the
  *     isotropic stencils the two segments are the lower and upper halves of a
  *     pair, both marching upwards, with sliding row sums;
  *   LF_VARIANT_SPLIT3 (3D default): three passes per step -- mu and F by a

@@ -357,7 +357,7 @@ inline int march_rows_for(int nx, int ny, int U, int param)
     return h;
 }
 
-// Rows per lane for the two-segment kernel.  Co-resident CTAs share an SM's
+// Rows per lane for the one-lane marches.  Co-resident CTAs share an SM's
 // issue rate, so the step takes about (CTAs per SM, rounded up) x (rows per
 // lane + 4 pipeline iterations); the smallest such cost wins among heights
 // that still give every SM about two CTAs (8 warps) when the lattice allows.
@@ -378,6 +378,56 @@ inline int march2_rows_for(int nx, int ny, int U, int param, int sms)
         const int lane = (ny + 2 * pairs - 1) / (2 * pairs);
         const int64_t cost = ((ctas + sms - 1) / sms) * (lane + 4);
         if (best_cost < 0 || cost < best_cost) { best_cost = cost; best = h; }
+    }
+    return best;
+}
+
+// CTA width and rows per lane of the two-lane (packed FP32) marches.  A CTA of
+// 64 threads (56 columns) or 128 (120) brings two or four warps, and an SM's
+// four schedulers take three warps each (six or three CTAs, by registers).
+// What counts is k, the warps per scheduler: two 64-thread CTAs per SM cost
+// what one of 128 threads does.  A pass of lanes of l rows with k = 1, 2, 3
+// takes about s_k l + c_k us, measured over 64^2 to 4096^2 at heights of 1 to
+// 120 rows and both widths (compact 1.10 / 1.24 / 1.89 us a row, isotropic
+// 1.33 / 1.70 / 2.15), full passes of k = 3 follow one another, and 3 us are
+// the launch.  The least sum wins; 64 threads cost about 2 % less at one k,
+// their blocks being halved finer at the same columns per warp.  The choice is
+// within 0.2 % of the best measured shape on average (2 % at worst); against
+// (CTAs per SM) x (l + 4) on 128 threads: 256^2 8.5 -> 7.4 us a step, 512^2
+// 13.4 -> 12.0, 1024^2 25.4 -> 24.4, isotropic 384^2 15.7 -> 13.1, 1024^2
+// 35.9 -> 32.8, 2999 x 1777 133.6 -> 120.  The tuner's param names a height
+// (low 16 bits) and 64 threads (bit 16); a height alone means 128 threads.
+struct PairShape {
+    bool narrow;                                    // 64 threads
+    int rows;
+};
+
+inline PairShape pair_shape(int nx, int ny, int tune, bool iso, int sms)
+{
+    const int fixed = tune & 0xFFFF, width = tune >> 16;
+    if (fixed > 0) return {width == 1, fixed < ny ? fixed : ny};
+    const float row[2][4] = {{0, 1.10f, 1.24f, 1.89f}, {0, 1.33f, 1.70f, 2.15f}};
+    const float lag[2][4] = {{0, 2.6f, 3.0f, 3.4f}, {0, 5.0f, 5.5f, 6.4f}};
+    PairShape best{width == 1, 1};
+    float best_us = -1.f;
+    for (int narrow = width == 1 ? 1 : 0; narrow < 2; ++narrow) {
+        const int U = narrow ? 56 : 120, strips = (nx + U - 1) / U;
+        for (int h = 1; h <= ny && h <= 512; ++h) {
+            int pairs = (ny + 2 * h - 1) / (2 * h);
+            if (pairs > ny / 2) pairs = ny / 2;     // every lane keeps at least one row
+            if (pairs < 1) break;
+            const int l = (ny + 2 * pairs - 1) / (2 * pairs);
+            const int64_t per_sm = ((int64_t)strips * pairs + sms - 1) / sms;
+            const int64_t k = narrow ? (per_sm + 1) / 2 : per_sm;
+            float us = 3.f + (float)(k / 3) * (row[iso][3] * l + lag[iso][3]);
+            if (k % 3) us += row[iso][k % 3] * l + lag[iso][k % 3];
+            if (narrow) us *= 0.98f;
+            if (best_us < 0.f || us < best_us) {
+                best_us = us;
+                best = {narrow == 1, h};
+            }
+            if (per_sm == 1) break;                 // taller lanes only take longer
+        }
     }
     return best;
 }

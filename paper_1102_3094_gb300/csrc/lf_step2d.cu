@@ -113,20 +113,17 @@ int spread_of(dim3 grid, int sms, int most = sizeof(R) == 4 ? 3 : 2)
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
-cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, cudaStream_t s)
+cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int H, int sms, cudaStream_t s)
 {
     using M = march::March2<NT, D>;
     auto kern = k_march2d_x2<NT, D, HYDRO, MINB>;
     static unsigned long long attr_done = 0;
-    cudaError_t e = raise_smem_limit(kern, (int)M::BYTES, &attr_done);
+    const cudaError_t e = raise_smem_limit(kern, (int)M::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
-    int sms = 0;
-    if ((e = device_sms(&sms)) != cudaSuccess) return e;
-    const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms), s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms, NT == 64 ? 6 : 3), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -145,20 +142,17 @@ cudaError_t launch_march(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
-cudaError_t launch_march_iso_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, cudaStream_t s)
+cudaError_t launch_march_iso_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int H, int sms, cudaStream_t s)
 {
     using M = march::MarchIso2<NT, D>;
     auto kern = k_march2d_iso_x2<NT, D, HYDRO, MINB>;
     static unsigned long long attr_done = 0;
-    cudaError_t e = raise_smem_limit(kern, (int)M::BYTES, &attr_done);
+    const cudaError_t e = raise_smem_limit(kern, (int)M::BYTES, &attr_done);
     if (e != cudaSuccess) return e;
-    int sms = 0;
-    if ((e = device_sms(&sms)) != cudaSuccess) return e;
-    const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms), s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms, NT == 64 ? 6 : 3), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -174,6 +168,27 @@ cudaError_t launch_march_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
     return launch_chained(kern, grid, NT, M::BYTES, spread_of<R>(grid, sms), s, g, p, io, H);
+}
+
+// The two-lane marches: width and rows per lane by march::pair_shape.
+template <bool HYDRO>
+cudaError_t launch_pair_shape(const Geom& g, const Phys<float>& p, const StepIO<float>& io, cudaStream_t s)
+{
+    int sms = 0;
+    const cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const bool iso = g.stencil == LF_STENCIL_ISOTROPIC;
+    const march::PairShape c = march::pair_shape(g.nx, g.ny, g.tune, iso, sms);
+    if (iso)
+        return c.narrow ? launch_march_iso_x2<64, 3, HYDRO, 6>(g, p, io, c.rows, sms, s)
+                        : launch_march_iso_x2<128, 3, HYDRO, 3>(g, p, io, c.rows, sms, s);
+    return c.narrow ? launch_march_x2<64, 3, HYDRO, 6>(g, p, io, c.rows, sms, s)
+                    : launch_march_x2<128, 3, HYDRO, 3>(g, p, io, c.rows, sms, s);
+}
+
+cudaError_t launch_pair(const Geom& g, const Phys<float>& p, const StepIO<float>& io, cudaStream_t s)
+{
+    return p.hydro ? launch_pair_shape<true>(g, p, io, s) : launch_pair_shape<false>(g, p, io, s);
 }
 
 template <typename R, int TX, int TY, int NT, bool AUX, bool ISO>
@@ -251,16 +266,10 @@ cudaError_t launch_step2d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, 
     if constexpr (sizeof(R) == 8) {
         if (!aux && g.variant == LF_VARIANT_MARCH && g.tune == 0 && f64_tiles(g)) return launch_step2d_f64(g, p, io, s);
     }
-    if (g.stencil == LF_STENCIL_ISOTROPIC) {           // the row marches or the tile kernel
-        if constexpr (sizeof(R) == 4) {
-            if (!aux && g.variant == LF_VARIANT_MARCH2 && g.ny >= 2) {
-                if ((g.tune >> 16) == 1)
-                    return p.hydro ? launch_march_iso_x2<64, 3, true, 6>(g, p, io, s)
-                                   : launch_march_iso_x2<64, 3, false, 6>(g, p, io, s);
-                return p.hydro ? launch_march_iso_x2<128, 3, true, 3>(g, p, io, s)
-                               : launch_march_iso_x2<128, 3, false, 3>(g, p, io, s);
-            }
-        }
+    if constexpr (sizeof(R) == 4) {
+        if (!aux && g.variant == LF_VARIANT_MARCH2 && g.ny >= 2) return launch_pair(g, p, io, s);
+    }
+    if (g.stencil == LF_STENCIL_ISOTROPIC) {           // the one-lane row march or the tile kernel
         if (!aux && (g.variant == LF_VARIANT_MARCH || g.variant == LF_VARIANT_MARCH2) && g.ny >= 2)
             return (g.tune >> 16) == 1 ? launch_march_iso<R, 64, 3>(g, p, io, s) : launch_march_iso<R, 128, 3>(g, p, io, s);
         if constexpr (sizeof(R) == 4)
@@ -269,15 +278,6 @@ cudaError_t launch_step2d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, 
         else
             return aux ? launch_cfg<R, 32, 16, 256, true, true>(g, p, io, s)
                        : launch_cfg<R, 32, 16, 256, false, true>(g, p, io, s);
-    }
-    if constexpr (sizeof(R) == 4) {
-        if (!aux && g.variant == LF_VARIANT_MARCH2 && g.ny >= 2)
-        {
-            if ((g.tune >> 16) == 1)
-                return p.hydro ? launch_march_x2<64, 3, true, 6>(g, p, io, s)
-                               : launch_march_x2<64, 3, false, 6>(g, p, io, s);
-            return p.hydro ? launch_march_x2<128, 3, true, 3>(g, p, io, s) : launch_march_x2<128, 3, false, 3>(g, p, io, s);
-        }
     }
     if (!aux && (g.variant == LF_VARIANT_MARCH || g.variant == LF_VARIANT_MARCH2))
         return (g.tune >> 16) == 1 ? launch_march<R, 64, 3>(g, p, io, s) : launch_march<R, 128, 3>(g, p, io, s);
