@@ -50,8 +50,9 @@ int lf_ens_create(int nruns, const lf_grid* grids, const lf_walls* walls, const 
  * the graphs. */
 int lf_ens_tune(lf_ens* e, int reps);
 
-/* Rows per segment the work list uses for run r (after tuning, or the
- * default min(16, ny / 2)). */
+/* Rows per segment the work list uses for run r: after tuning, or the default,
+ * one height for all runs of a stencil (at most ny / 2) chosen from their
+ * sizes, their number and the SM count. */
 int lf_ens_rows(const lf_ens* e, int run);
 
 /* The LF_VARIANT_MARCH2 param of run r's shape: (1 << 16 for 64-thread CTAs,

@@ -5,8 +5,8 @@
 // a work list of (run, strip, pair) items -- each item is exactly the
 // two-lane row-marching step of lf_march2d_x2.cuh (two segments of a strip
 // marching away from their common row) -- followed, when some runs need extra
-// temperature sub-steps, by one launch per sub-step over the tiles of those
-// runs.  Runs with the isotropic stencils are (run, strip, pair) items of a
+// temperature sub-steps, by one launch per up to four of them (lf_tsub2d.cuh)
+// over the strips and row segments of those runs.  Runs with the isotropic stencils are (run, strip, pair) items of a
 // second persistent kernel that runs the two-lane isotropic row march
 // (lf_march2d_iso.cuh), the code a single isotropic FP32 run uses by default.
 // Every run returns to its starting buffers
@@ -27,7 +27,7 @@
 #include "lf_ens.h"
 #include "lf_march2d_iso.cuh"
 #include "lf_march2d_x2.cuh"
-#include "lf_tile2d.cuh"
+#include "lf_tsub2d.cuh"
 
 using namespace lf;
 
@@ -60,7 +60,7 @@ struct EnsT {
 };
 
 struct EnsTItem {
-    int run, bx, by;
+    int run, strip, y0, y1, n;      // n sub-steps at once on rows y0 .. y1 - 1
 };
 
 // Isotropic runs: (run, strip, pair) items of the two-lane isotropic march,
@@ -116,20 +116,36 @@ int pairs_for(int ny, int H)
     return np < 1 ? 1 : np;
 }
 
-__global__ void __launch_bounds__(256) k_ens_tsub2d(const EnsT* __restrict__ runs, const EnsTItem* __restrict__ items,
+// The next one to four temperature sub-steps of every run that has any left:
+// a warp per (run, strip, row segment), the passes of lf_step on a single run.
+// Bound by the latency of a segment's march (its rows and 2 n more); one launch
+// for up to four sub-steps takes 22 us for 96 runs of 128^2 to 512^2 with xi up
+// to 1, one launch for each of the four 33 us (caches cold).
+__global__ void __launch_bounds__(128) k_ens_tsub2d(const EnsT* __restrict__ runs, const EnsTItem* __restrict__ items,
                                                    int nitems)
 {
-    chain_next();
     chain_wait();
-    for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
+    const int it = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (it < nitems) {                              // for the whole warp
         const EnsTItem w = items[it];
         const EnsT r = runs[w.run];
-        const int x = w.bx * 32 + (threadIdx.x & 31), y = w.by * 8 + (threadIdx.x >> 5);
-        if (x < r.g.nx && y < r.g.ny) {
-            if (r.g.stencil == LF_STENCIL_ISOTROPIC) tile::tsub2d_site_iso(r.g, r.p, r.Tin, r.Tout, x, y);
-            else march::tsub2d_site(r.g, r.p, r.Tin, r.Tout, x, y);
+        if (r.g.stencil == LF_STENCIL_ISOTROPIC) {
+            switch (w.n) {
+            case 1: tsub::tsub2d_rows<1, true>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            case 2: tsub::tsub2d_rows<2, true>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            case 3: tsub::tsub2d_rows<3, true>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            default: tsub::tsub2d_rows<4, true>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            }
+        } else {
+            switch (w.n) {
+            case 1: tsub::tsub2d_rows<1, false>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            case 2: tsub::tsub2d_rows<2, false>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            case 3: tsub::tsub2d_rows<3, false>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            default: tsub::tsub2d_rows<4, false>(r.g, r.p, r.Tin, r.Tout, w.strip, w.y0, w.y1); break;
+            }
         }
     }
+    chain_next();
 }
 
 Phys<float> phys_f(const lf_ctx* c)
@@ -146,6 +162,14 @@ Phys<float> phys_f(const lf_ctx* c)
     ph.n0 = (float)p.n0;
     ph.hydro = p.hydro;
     return ph;
+}
+
+// Sub-steps of each pass after a run's step kernel.
+std::vector<int> tsub_passes(const lf_ctx* c, bool t_update)
+{
+    std::vector<int> v;
+    for (int left = t_update ? c->nsub - 1 : 0; left > 0; left -= v.back()) v.push_back(tsub_fused<float>(c->g, left));
+    return v;
 }
 
 struct Cursor {
@@ -168,6 +192,7 @@ struct lf_ens {
     int parity;                     // 0: the next step is step A of the cycle, 1: step B
     std::vector<Cursor> base;       // buffer cursors at the start of step A
     int march_blocks[4];            // 64- and 128-thread march kernels, compact then isotropic
+    int spread[4];                  // CTAs per SM an even spread of them needs, 0 when the SMs are full
     int nitems[4];
     EnsItem* d_items[4];
 };
@@ -187,7 +212,7 @@ void free_graphs(lf_ens* e)
 // Device layout of one half-cycle (step A or B): run table, T tables.
 struct Half {
     EnsRun* runs;
-    std::vector<EnsT*> ts;          // per extra sub-step s = 1 .. max_nsub - 1
+    std::vector<EnsT*> ts;          // per pass of extra sub-steps
 };
 
 int capture(lf_ens* e, const std::vector<int>& halves, const Half* H, const std::vector<EnsTItem*>& titems,
@@ -197,21 +222,20 @@ int capture(lf_ens* e, const std::vector<int>& halves, const Half* H, const std:
     if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LF_ECUDA;
     for (int h : halves) {
         if (e->nitems[0] > 0)
-            launch_chained(kEns64, e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->stream, H[h].runs, e->d_items[0],
-                           e->nitems[0]);
+            launch_chained(kEns64, e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->spread[0], e->stream, H[h].runs,
+                           e->d_items[0], e->nitems[0]);
         if (e->nitems[1] > 0)
-            launch_chained(kEns128, e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->stream, H[h].runs, e->d_items[1],
-                           e->nitems[1]);
+            launch_chained(kEns128, e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->spread[1], e->stream, H[h].runs,
+                           e->d_items[1], e->nitems[1]);
         if (e->nitems[2] > 0)
-            launch_chained(kIso64, e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->stream, H[h].runs, e->d_items[2],
-                           e->nitems[2]);
+            launch_chained(kIso64, e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->spread[2], e->stream, H[h].runs,
+                           e->d_items[2], e->nitems[2]);
         if (e->nitems[3] > 0)
-            launch_chained(kIso128, e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->stream, H[h].runs, e->d_items[3],
-                           e->nitems[3]);
+            launch_chained(kIso128, e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->spread[3], e->stream, H[h].runs,
+                           e->d_items[3], e->nitems[3]);
         for (size_t s = 0; s < H[h].ts.size(); ++s) {
             if (ntitems[s] == 0) continue;
-            const int blocks = std::min(ntitems[s], 152 * 8);
-            launch_chained(k_ens_tsub2d, blocks, 256, 0, e->stream, H[h].ts[s], titems[s], ntitems[s]);
+            launch_chained(k_ens_tsub2d, (ntitems[s] + 3) / 4, 128, 0, e->stream, H[h].ts[s], titems[s], ntitems[s]);
         }
     }
     cudaError_t err = cudaStreamEndCapture(e->stream, &graph);   // reports a failed launch too
@@ -227,9 +251,16 @@ int build(lf_ens* e)
 {
     free_graphs(e);
     const int R = e->nruns;
-    int max_nsub = 1;
-    for (lf_ctx* c : e->runs)
-        if (phys_f(c).t_update) max_nsub = std::max(max_nsub, c->nsub);
+    int npass = 0;
+    std::vector<std::vector<int>> passes(R);
+    for (int r = 0; r < R; ++r) {
+        passes[r] = tsub_passes(e->runs[r], phys_f(e->runs[r]).t_update);
+        npass = std::max(npass, (int)passes[r].size());
+    }
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
 
     // host tables for both halves
     e->base.resize(R);
@@ -237,7 +268,7 @@ int build(lf_ens* e)
     std::vector<std::vector<EnsT>> ht[2];
     for (int h = 0; h < 2; ++h) {
         hr[h].resize(R);
-        ht[h].assign(max_nsub - 1, std::vector<EnsT>(R));
+        ht[h].assign(npass, std::vector<EnsT>(R));
     }
     for (int r = 0; r < R; ++r) {
         lf_ctx* c = e->runs[r];
@@ -259,13 +290,13 @@ int build(lf_ens* e)
             if (c->params.hydro) cur.f ^= 1;
             cur.p ^= 1;
             cur.t ^= 1;
-            for (int s = 1; s < max_nsub; ++s) {
-                EnsT& t = ht[h][s - 1][r];
+            for (int s = 0; s < npass; ++s) {
+                EnsT& t = ht[h][s][r];
                 t.g = c->g;
                 t.p = ph;
                 t.Tin = (const float*)c->T[cur.t];
                 t.Tout = (float*)c->T[cur.t ^ 1];
-                if (ph.t_update && s < c->nsub) cur.t ^= 1;
+                if (s < (int)passes[r].size()) cur.t ^= 1;
             }
         }
     }
@@ -290,19 +321,30 @@ int build(lf_ens* e)
     };
     for (auto& it : items)
         std::stable_sort(it.begin(), it.end(), [&](const EnsItem& a, const EnsItem& b) { return lane(a) > lane(b); });
-    std::vector<std::vector<EnsTItem>> titems(max_nsub > 1 ? max_nsub - 1 : 0);
-    for (int s = 1; s < max_nsub; ++s)
+    std::vector<std::vector<EnsTItem>> titems(npass);
+    for (int s = 0; s < npass; ++s) {
+        // about sixteen warps per SM in all, segments of 4 to 64 rows, the
+        // longest first
+        auto strips_of = [&](int r) { return ((e->runs[r]->g.nx + 3) / 4 + tsub::kQuads - 1) / tsub::kQuads; };
+        auto due = [&](int r) { return e->active[r] && s < (int)passes[r].size(); };
+        int64_t rows = 0;
+        for (int r = 0; r < R; ++r)
+            if (due(r)) rows += (int64_t)strips_of(r) * e->runs[r]->g.ny;
+        const int H = (int)std::min<int64_t>(64, std::max<int64_t>(4, (rows + 16 * sms - 1) / (16 * sms)));
         for (int r = 0; r < R; ++r) {
-            const lf_ctx* c = e->runs[r];
-            if (!e->active[r] || !phys_f(c).t_update || s >= c->nsub) continue;
-            for (int by = 0; by < (c->g.ny + 7) / 8; ++by)
-                for (int bx = 0; bx < (c->g.nx + 31) / 32; ++bx) titems[s - 1].push_back({r, bx, by});
+            const int ny = e->runs[r]->g.ny;
+            if (due(r))
+                for (int y0 = 0; y0 < ny; y0 += H)
+                    for (int st = 0; st < strips_of(r); ++st)
+                        titems[s].push_back({r, st, y0, std::min(y0 + H, ny), passes[r][s]});
         }
+        std::stable_sort(titems[s].begin(), titems[s].end(), [](const EnsTItem& a, const EnsTItem& b) { return a.n > b.n; });
+    }
     // one device block for everything
     auto a256 = [](size_t v) { return (v + 255) / 256 * 256; };
     size_t bytes = 2 * a256(sizeof(EnsRun) * R);
     for (const auto& it : items) bytes += a256(sizeof(EnsItem) * it.size());
-    for (int s = 1; s < max_nsub; ++s) bytes += 2 * a256(sizeof(EnsT) * R) + a256(sizeof(EnsTItem) * titems[s - 1].size());
+    for (int s = 0; s < npass; ++s) bytes += 2 * a256(sizeof(EnsT) * R) + a256(sizeof(EnsTItem) * titems[s].size());
     if (cudaMalloc((void**)&e->tables, bytes) != cudaSuccess) { cudaGetLastError(); return LF_ENOMEM; }
     unsigned char* p = e->tables;
     Half halves[2];
@@ -320,16 +362,16 @@ int build(lf_ens* e)
     }
     std::vector<EnsTItem*> d_titems;
     std::vector<int> ntitems;
-    for (int s = 1; s < max_nsub; ++s) {
+    for (int s = 0; s < npass; ++s) {
         for (int h = 0; h < 2; ++h) {
             halves[h].ts.push_back((EnsT*)p);
-            copies.push_back({p, {ht[h][s - 1].data(), sizeof(EnsT) * R}});
+            copies.push_back({p, {ht[h][s].data(), sizeof(EnsT) * R}});
             p += a256(sizeof(EnsT) * R);
         }
         d_titems.push_back((EnsTItem*)p);
-        ntitems.push_back((int)titems[s - 1].size());
-        copies.push_back({p, {titems[s - 1].data(), sizeof(EnsTItem) * titems[s - 1].size()}});
-        p += a256(sizeof(EnsTItem) * titems[s - 1].size());
+        ntitems.push_back((int)titems[s].size());
+        copies.push_back({p, {titems[s].data(), sizeof(EnsTItem) * titems[s].size()}});
+        p += a256(sizeof(EnsTItem) * titems[s].size());
     }
     for (auto& cp : copies)
         if (cp.second.second && cudaMemcpyAsync(cp.first, cp.second.first, cp.second.second, cudaMemcpyHostToDevice,
@@ -347,15 +389,16 @@ int build(lf_ens* e)
         cudaFuncSetAttribute(kIso128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)IsoCfg<128>::BYTES) !=
             cudaSuccess)
         return LF_ECUDA;
-    int per_sm[4] = {0, 0, 0, 0}, sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int per_sm[4] = {0, 0, 0, 0};
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], kEns64, 64, MarchCfg<64>::BYTES);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], kEns128, 128, MarchCfg<128>::BYTES);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], kIso64, 64, IsoCfg<64>::BYTES);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[3], kIso128, 128, IsoCfg<128>::BYTES);
-    for (int wi = 0; wi < 4; ++wi)
-        e->march_blocks[wi] = std::max(1, std::min(e->nitems[wi], std::max(1, per_sm[wi]) * std::max(1, sms)));
+    for (int wi = 0; wi < 4; ++wi) {
+        e->march_blocks[wi] = std::max(1, std::min(e->nitems[wi], std::max(1, per_sm[wi]) * sms));
+        const int k = (e->march_blocks[wi] + sms - 1) / sms;
+        e->spread[wi] = k < per_sm[wi] ? k : 0;
+    }
 
     if ((rc = capture(e, {0}, halves, d_titems, ntitems, &e->gA)) != LF_OK) return rc;
     if ((rc = capture(e, {1}, halves, d_titems, ntitems, &e->gB)) != LF_OK) return rc;
@@ -364,13 +407,68 @@ int build(lf_ens* e)
     return LF_OK;
 }
 
+// Rows per lane of every run before any tuning, one height for all runs of a
+// stencil, with 64-thread CTAs (the better width at 4 to 96 runs of 128^2 to
+// 512^2, both stencils).  Six CTAs fit an SM; CTA b takes the items b, b + B,
+// ... of the list sorted by length, so the step takes what CTA 0 does: per
+// item of l rows about s l + c us, measured with heights of 2 to 128 (compact
+// 1.89 l + 5.5, isotropic 2.4 l + 10; s falls to 1.24 / 1.7 and 1.1 / 1.33
+// where four or two CTAs per SM hold all items).  Against 16 rows: 10 runs 45.6
+// -> 41.3 us a step, 48 runs 168 -> 149, 96 runs 313 -> 273, isotropic 411 ->
+// 354; within 1 % of the best uniform height at seven of eight counts of runs.
+void default_rows(lf_ens* e)
+{
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    sms = std::max(1, sms);
+    const float row[2][4] = {{0, 1.10f, 1.24f, 1.89f}, {0, 1.33f, 1.70f, 2.4f}};
+    const float lag[2] = {5.5f, 10.f};
+    for (int iso = 0; iso < 2; ++iso) {
+        std::vector<int> members;
+        int tallest = 0;
+        for (int r = 0; r < e->nruns; ++r) {
+            const Geom& g = e->runs[r]->g;
+            if ((g.stencil == LF_STENCIL_ISOTROPIC) != (iso == 1)) continue;
+            members.push_back(r);
+            tallest = std::max(tallest, g.ny);
+        }
+        if (members.empty()) continue;
+        int best = 1;
+        float best_us = -1.f;
+        std::vector<std::pair<int, int64_t>> lanes(members.size());      // rows per lane, items
+        for (int h = 1; h <= std::max(1, tallest / 2) && h <= 512; ++h) {
+            int64_t items = 0;
+            for (size_t m = 0; m < members.size(); ++m) {
+                const Geom& g = e->runs[members[m]]->g;
+                const int np = pairs_for(g.ny, h);
+                lanes[m] = {(g.ny + 2 * np - 1) / (2 * np), (int64_t)np * ((g.nx + MarchCfg<64>::U - 1) / MarchCfg<64>::U)};
+                items += lanes[m].second;
+            }
+            std::sort(lanes.begin(), lanes.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
+            const int64_t B = std::min<int64_t>(items, 6 * (int64_t)sms);
+            const int k = (int)std::min<int64_t>(3, ((B + sms - 1) / sms + 1) / 2);
+            float us = 0.f;
+            int64_t next = 0, end = 0;                                   // CTA 0's next item; items seen
+            for (const auto& l : lanes) {
+                end += l.second;
+                for (; next < end; next += B) us += row[iso][k] * l.first + lag[iso];
+            }
+            if (best_us < 0.f || us < best_us) {
+                best_us = us;
+                best = h;
+            }
+        }
+        for (int r : members) e->rows[r] = std::max(1, std::min(best, e->runs[r]->g.ny / 2));
+    }
+}
+
 void advance_cursors(lf_ens* e, int64_t n)
 {
     for (size_t r = 0; r < e->runs.size(); ++r) {
         if (!e->active[r]) continue;
         lf_ctx* c = e->runs[r];
-        const bool tu = phys_f(c).t_update;
-        const int tflips = tu ? c->nsub : 1;
+        const int tflips = 1 + (int)tsub_passes(c, phys_f(c).t_update).size();
         if ((n & 1) != 0) {
             if (c->params.hydro) c->fcur ^= 1;
             c->pcur ^= 1;
@@ -431,12 +529,15 @@ int lf_ens_create(int nruns, const lf_grid* grids, const lf_walls* walls, const 
         if (rc == LF_OK) {
             c->ens_member = true;
             e->runs.push_back(c);
-            e->rows.push_back(c->g.ny / 2 < 16 ? (c->g.ny / 2 > 0 ? c->g.ny / 2 : 1) : 16);
+            e->rows.push_back(1);
             e->width.push_back(64);
             e->active.push_back(1);
         }
     }
-    if (rc == LF_OK) rc = build(e);
+    if (rc == LF_OK) {
+        default_rows(e);
+        rc = build(e);
+    }
     if (rc != LF_OK) {
         lf_ens_destroy(e);
         return rc;
@@ -487,9 +588,14 @@ int lf_ens_tune(lf_ens* e, int reps)
                 x->rows[r] = h;
             }
     };
-    const int cand[] = {1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128};
     for (const auto& key : keys) {
         const int ny = std::get<1>(key);
+        std::vector<int> cand{1, 2, 3, 4, 6, 8, 12, 16, 24, 32, 48, 64, 96, 128};
+        for (int r = 0; r < R; ++r)                  // and the present height
+            if (key_of(e->runs[r]) == key && std::find(cand.begin(), cand.end(), e->rows[r]) == cand.end()) {
+                cand.push_back(e->rows[r]);
+                break;
+            }
         float best_ms = 1e30f;
         std::pair<int, int> best_wh{64, 16};
         for (int w : {64, 128})
