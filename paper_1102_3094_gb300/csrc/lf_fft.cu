@@ -16,10 +16,12 @@
 //     and a CTA keeps them (and the digit reversal) over all its lines.
 // 256^3, one axis: 985 us before; now 360 us along y (the pipe's time for 22
 // operations per point of the half spectrum: 354 us), 412 us along x from the
-// field, 528 us back to it.
+// field, 448 us back to it (528 with the scaling, the test for finite values and
+// the narrowing on the FP64 pipe).
 #include <algorithm>
 #include <cmath>
 
+#include "lf_cvt.h"
 #include "lf_fft.cuh"
 
 namespace lf {
@@ -127,6 +129,15 @@ __device__ __noinline__ void dft_any(double2* x, int r, const double2* tw, int w
     for (int q = 0; q < r; ++q) x[q] = y[q];
 }
 
+// Stores off the FP64 pipe (lf_cvt.h): no conversion, no comparison on it.
+__device__ __forceinline__ void narrow(double v, float* p)
+{
+    uint32_t b;
+    *p = narrow_bits((uint64_t)__double_as_longlong(v), &b) ? __uint_as_float(b) : (float)v;
+}
+__device__ __forceinline__ void narrow(double v, double* p) { *p = v; }
+__device__ __forceinline__ bool finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
 // Quotient and remainder by d: shifts when the line length is a power of two
 // (then d is one too), else a division.
 template <bool POW2>
@@ -190,7 +201,6 @@ template <typename R>
 struct RealOut {
     const double2* in;
     R* f;
-    double scale;
     int64_t rows;
     int pitch;
     static constexpr bool kAlongLine = true;
@@ -207,12 +217,11 @@ struct RealOut {
     __device__ __forceinline__ bool store(int64_t, int64_t l, int j, int, const double2* buf) const
     {
         const double2 v = buf[j];
-        const double a = v.x * scale, b = v.y * scale;
         R* p = f + 2 * l * pitch + j;
-        p[0] = (R)a;
-        if (2 * l + 1 >= rows) return isfinite(a);
-        p[pitch] = (R)b;
-        return isfinite(a) && isfinite(b);
+        narrow(v.x, p);
+        if (2 * l + 1 >= rows) return finite(v.x);
+        narrow(v.y, p + pitch);
+        return finite(v.x) && finite(v.y);
     }
 };
 
@@ -418,15 +427,15 @@ cudaError_t fft_axis(const Geom& g, double2* data, int axis, cudaStream_t s)
 }
 
 template <typename R>
-cudaError_t irfft_x(const Geom& g, const double2* in, double scale, R* f, int* flag, cudaStream_t s)
+cudaError_t irfft_x(const Geom& g, const double2* in, R* f, int* flag, cudaStream_t s)
 {
     const int64_t rows = (int64_t)g.ny * g.nz;
-    return run_lines(RealOut<R>{in, f, scale, rows, g.pitch}, g.nx, (rows + 1) / 2, flag, s);
+    return run_lines(RealOut<R>{in, f, rows, g.pitch}, g.nx, (rows + 1) / 2, flag, s);
 }
 
 #define LF_INST(R)                                                                       \
     template cudaError_t rfft_x<R>(const Geom&, const R*, double2*, cudaStream_t);       \
-    template cudaError_t irfft_x<R>(const Geom&, const double2*, double, R*, int*, cudaStream_t);
+    template cudaError_t irfft_x<R>(const Geom&, const double2*, R*, int*, cudaStream_t);
 LF_INST(float)
 LF_INST(double)
 #undef LF_INST

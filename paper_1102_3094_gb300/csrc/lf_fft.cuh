@@ -25,10 +25,10 @@ cudaError_t rfft_x(const Geom& g, const R* f, double2* out, cudaStream_t s);
 // Forward DFT along axis 1 (y) or 2 (z) of a half spectrum, in place.
 cudaError_t fft_axis(const Geom& g, double2* data, int axis, cudaStream_t s);
 
-// f = scale x DFT along x of the half spectrum `in`, whose rows are the DFTs
-// of real rows up to a conjugation (so the result is real).  Sets *flag when a
-// value is not finite.
+// f = DFT along x of the half spectrum `in`, whose rows are the DFTs of real
+// rows up to a conjugation (so the result is real).  Sets *flag when a value is
+// not finite.
 template <typename R>
-cudaError_t irfft_x(const Geom& g, const double2* in, double scale, R* f, int* flag, cudaStream_t s);
+cudaError_t irfft_x(const Geom& g, const double2* in, R* f, int* flag, cudaStream_t s);
 
 }  // namespace lf

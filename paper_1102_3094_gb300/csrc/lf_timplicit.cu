@@ -126,11 +126,12 @@ __device__ __forceinline__ double tri_diag(const TriSys& t, int j, int t_mode)
 }
 
 // The part of the Thomas algorithm that does not depend on the right-hand
-// side: c'_j = a / (b_j - a c'_{j-1}) and the reciprocal pivot
-// 1 / (b_j - a c'_{j-1}) of every unknown layer of every mode, stored at
+// side: c'_j = a / (b_j - a c'_{j-1}) and the scaled reciprocal pivot
+// scale / (b_j - a c'_{j-1}) of every unknown layer of every mode, stored at
 // j * M + m (c') and N + j * M + m (pivot).  The coefficients do not change
-// from step to step, so the divisions leave the per-step recurrence.
-__global__ void k_t_coef(Geom g, double* __restrict__ coef, double xi, int t_mode)
+// from step to step, so the divisions leave the per-step recurrence, and the
+// transforms' normalisation costs nothing there.
+__global__ void k_t_coef(Geom g, double* __restrict__ coef, double xi, int t_mode, double scale)
 {
     const int d = g.d;
     const int64_t M = wall_modes(g);
@@ -144,7 +145,7 @@ __global__ void k_t_coef(Geom g, double* __restrict__ coef, double xi, int t_mod
         const double inv = 1.0 / (tri_diag(t, j, t_mode) - t.a * cprev);
         const double cj = t.a * inv;
         coef[(int64_t)j * M + m] = cj;
-        coef[N + (int64_t)j * M + m] = inv;
+        coef[N + (int64_t)j * M + m] = inv * scale;
         cprev = cj;
     }
 }
@@ -152,10 +153,14 @@ __global__ void k_t_coef(Geom g, double* __restrict__ coef, double xi, int t_mod
 // Walls along the last axis: one thread per Fourier mode m of the periodic
 // axes (M modes), the Thomas sweeps along the L layers of the wall normal
 // with c' and the pivots from k_t_coef; element (j, m) at j * M + m.  The
-// serial chain holds only multiply-adds: dp_j = (d_j - a dp_{j-1}) pivot_j,
-// x_j = dp_j - c'_j x_{j+1}.  Writes the conjugate of the solution.
+// serial chain holds only multiply-adds: dp_j = (d_j - a / scale dp_{j-1})
+// pivot_j, x_j = dp_j - c'_j x_{j+1}.  Writes scale times the conjugate of the
+// solution.  Bound by memory and the FP64 pipe alike (256^3: 675 MB, 100 us, and
+// 97 us of operations in 181 us); two threads per mode (193 us), fewer CTAs at a
+// time so that a wave stays in the L2 (226 to 361 us) and prefetches further
+// ahead (196 us) were no better.
 __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __restrict__ coef, double xi,
-                           double Tw_hat0, int t_mode)
+                           double Tw_hat0, int t_mode, double scale)
 {
     const int d = g.d;
     const int64_t M = wall_modes(g);
@@ -164,7 +169,7 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
     const int64_t m = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (m >= M) return;
     const TriSys t = tri_sys(g, m, xi, t_mode, L);
-    const double a = t.a;
+    const double a = t.a, as = a / scale;
     const int j0 = t.j0, j1 = t.j1;
     auto at = [&](int j) -> double2& { return buf[(int64_t)j * M + m]; };
     double2 lo_add, hi_add;
@@ -177,7 +182,7 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
         hi_add = make_double2(w, 0.0);
     }
     if (j1 < j0) {                           // no unknown layer
-        for (int j = 0; j < L; ++j) at(j) = make_double2(at(j).x, -at(j).y);
+        for (int j = 0; j < L; ++j) at(j) = make_double2(scale * at(j).x, -scale * at(j).y);
         return;
     }
     // Forward sweep in blocks of kB layers: the right-hand sides and pivots of
@@ -205,7 +210,7 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
             double2 dj = dv[u];
             if (j == j0) { dj.x += lo_add.x; dj.y += lo_add.y; }
             if (j == j1) { dj.x += hi_add.x; dj.y += hi_add.y; }
-            const double2 dp = make_double2((dj.x - a * dprev.x) * pv[u], (dj.y - a * dprev.y) * pv[u]);
+            const double2 dp = make_double2((dj.x - as * dprev.x) * pv[u], (dj.y - as * dprev.y) * pv[u]);
             at(j) = dp;
             dprev = dp;
         }
@@ -235,16 +240,17 @@ __global__ void k_t_thomas(Geom g, double2* __restrict__ buf, const double* __re
 #pragma unroll
         for (int u = 0; u < kB; ++u) { dv[u] = dn[u]; pv[u] = pn[u]; }
     }
-    for (int j = 0; j < j0; ++j) at(j) = make_double2(at(j).x, -at(j).y);          // held layers
-    for (int j = j1 + 1; j < L; ++j) at(j) = make_double2(at(j).x, -at(j).y);
+    for (int j = 0; j < j0; ++j) at(j) = make_double2(scale * at(j).x, -scale * at(j).y);          // held layers
+    for (int j = j1 + 1; j < L; ++j) at(j) = make_double2(scale * at(j).x, -scale * at(j).y);
 }
 
-// Every axis periodic: the mode is divided by 1 + xi lam; writes the conjugate.
-__global__ void k_t_divide(Geom g, double2* __restrict__ buf, double xi)
+// Every axis periodic: the mode is divided by 1 + xi lam; writes scale times the
+// conjugate.
+__global__ void k_t_divide(Geom g, double2* __restrict__ buf, double xi, double scale)
 {
     const int64_t N = (int64_t)half_nx(g.nx) * g.ny * g.nz;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const double s = 1.0 / (1.0 + xi * lam_periodic(g, k));
+        const double s = scale / (1.0 + xi * lam_periodic(g, k));
         buf[k] = make_double2(buf[k].x * s, -buf[k].y * s);
     }
 }
@@ -277,7 +283,9 @@ int t_implicit_step(lf_ctx* c, double xi, double T_w)
     int64_t nper = g.nx;
     if (nper_axes >= 2) nper *= g.ny;
     if (nper_axes >= 3) nper *= g.nz;
-    // the transform along x is taken from T itself and gives twice the half spectrum
+    // the transform along x is taken from T itself and gives twice the half
+    // spectrum; the solve takes the normalisation out of it
+    const double scale = 0.5 / (double)nper;
     if (rfft_x<R>(g, T, buf, s) != cudaSuccess) return LF_ECUDA;
     for (int a = 1; a < nper_axes; ++a)
         if (fft_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
@@ -285,20 +293,21 @@ int t_implicit_step(lf_ctx* c, double xi, double T_w)
         const int64_t M = wall_modes(g);
         if (!c->tcoef) return LF_EINVAL;     // lf_set_t_solver allocates the tables
         if (!c->tcoef_valid || c->tcoef_xi != xi || c->tcoef_mode != g.t_mode || c->tcoef_stencil != g.stencil) {
-            k_t_coef<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, c->tcoef, xi, g.t_mode);
+            k_t_coef<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, c->tcoef, xi, g.t_mode, scale);
             c->tcoef_valid = true;
             c->tcoef_xi = xi;
             c->tcoef_mode = g.t_mode;
             c->tcoef_stencil = g.stencil;
         }
-        k_t_thomas<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, buf, c->tcoef, xi, 2.0 * T_w * (double)nper, g.t_mode);
+        k_t_thomas<<<(unsigned)((M + 31) / 32), 32, 0, s>>>(g, buf, c->tcoef, xi, 2.0 * T_w * (double)nper, g.t_mode,
+                                                               scale);
     } else {
-        k_t_divide<<<grid_t((int64_t)half_nx(g.nx) * g.ny * g.nz), 256, 0, s>>>(g, buf, xi);
+        k_t_divide<<<grid_t((int64_t)half_nx(g.nx) * g.ny * g.nz), 256, 0, s>>>(g, buf, xi, scale);
     }
     if (cudaGetLastError() != cudaSuccess) return LF_ECUDA;
     for (int a = 1; a < nper_axes; ++a)
         if (fft_axis(g, buf, a, s) != cudaSuccess) return LF_ECUDA;
-    return irfft_x<R>(g, buf, 0.5 / (double)nper, T, c->flag_dev, s) == cudaSuccess ? LF_OK : LF_ECUDA;
+    return irfft_x<R>(g, buf, T, c->flag_dev, s) == cudaSuccess ? LF_OK : LF_ECUDA;
 }
 
 template int t_implicit_step<float>(lf_ctx*, double, double);
