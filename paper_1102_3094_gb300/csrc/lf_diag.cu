@@ -24,7 +24,8 @@ namespace lf {
 
 namespace {
 
-constexpr int kBlocks = 152 * 8;   // partial sums: a few waves on 152 SMs
+constexpr int kBlocks = 152 * 8;   // partial sums there is room for
+constexpr int kResident = 152 * 3; // CTAs of k_diag_partial that run at once
 constexpr int kThreads = 256;
 constexpr int kMaxBins = 2048;     // of S(k): half the longest line the FFT takes
 
@@ -68,95 +69,112 @@ __device__ __forceinline__ double at(const R* f, const Geom& g, int x, int y, in
     return (double)f[((int64_t)z * g.ny + y) * g.pitch + x];
 }
 
-// Central differences and the Laplacian of phi at (x, y, z); along the wall
-// axis the neighbour beyond the last layer is the layer itself (even mirror).
-// With `links` given, also the sum over the site's forward links of
-// (phi(r + e) - phi(r))^2: the mirror neighbour makes the link out of the
-// last layer vanish, so every nearest-neighbour link inside the lattice is
-// counted once.
+// Central differences of phi at (x, y, z); along the wall axis the neighbour
+// beyond the last layer is the layer itself (even mirror).
 template <typename R>
-__device__ void phi_derivs(const R* phi, const Geom& g, int x, int y, int z, double* grad, double* lap,
-                           double* links = nullptr)
+__device__ void phi_grad(const R* phi, const Geom& g, int x, int y, int z, double* grad)
 {
     const int wy = g.walls && g.d == 2, wz = g.walls && g.d == 3;
-    const double c = at(phi, g, x, y, z);
-    const double xp = at(phi, g, nb_index(x, 1, g.nx, 0), y, z), xm = at(phi, g, nb_index(x, -1, g.nx, 0), y, z);
-    const double yp = at(phi, g, x, nb_index(y, 1, g.ny, wy), z), ym = at(phi, g, x, nb_index(y, -1, g.ny, wy), z);
-    grad[0] = 0.5 * (xp - xm);
-    grad[1] = 0.5 * (yp - ym);
-    double l = xp + xm - 2.0 * c + yp + ym - 2.0 * c;
-    double k2 = (xp - c) * (xp - c) + (yp - c) * (yp - c);
+    grad[0] = 0.5 * (at(phi, g, nb_index(x, 1, g.nx, 0), y, z) - at(phi, g, nb_index(x, -1, g.nx, 0), y, z));
+    grad[1] = 0.5 * (at(phi, g, x, nb_index(y, 1, g.ny, wy), z) - at(phi, g, x, nb_index(y, -1, g.ny, wy), z));
     grad[2] = 0.0;
-    if (g.d == 3) {
-        const double zp = at(phi, g, x, y, nb_index(z, 1, g.nz, wz)), zm = at(phi, g, x, y, nb_index(z, -1, g.nz, wz));
-        grad[2] = 0.5 * (zp - zm);
-        l += zp + zm - 2.0 * c;
-        k2 += (zp - c) * (zp - c);
-    }
-    *lap = l;
-    if (links) *links = k2;
+    if (g.d == 3)
+        grad[2] = 0.5 * (at(phi, g, x, y, nb_index(z, 1, g.nz, wz)) - at(phi, g, x, y, nb_index(z, -1, g.nz, wz)));
 }
 
+// Sums (slot max_slot: maximum) of v over the CTA, in a fixed order.  The
+// values go through shared memory and 16 threads per slot add 16 of them each:
+// a fifth of the FP64 operations of a shuffle tree in every warp.
 template <int NQ>
 __device__ void block_reduce_store(double (&v)[NQ], double* out, int max_slot)
 {
-    __shared__ double red[kThreads / 32][NQ];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    static_assert(NQ % 2 == 0 && NQ * 16 <= kThreads && kThreads == 256, "whole warps of 16-thread groups");
+    __shared__ double red[NQ][kThreads];
+    const int tid = threadIdx.x;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        double x = v[q];
-        for (int o = 16; o > 0; o >>= 1) {
-            const double y = __shfl_down_sync(0xffffffffu, x, o);
-            x = (q == max_slot) ? fmax(x, y) : x + y;
-        }
-        if (lane == 0) red[warp][q] = x;
-    }
+    for (int q = 0; q < NQ; ++q) red[q][tid] = v[q];
     __syncthreads();
-    if (warp == 0) {
+    if (tid < NQ * 16) {
+        const int q = tid >> 4, l = tid & 15;
+        const bool mx = q == max_slot;
+        double x = red[q][l];
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-            double x = lane < kThreads / 32 ? red[lane][q] : (q == max_slot ? 0.0 : 0.0);
-            for (int o = 16; o > 0; o >>= 1) {
-                const double y = __shfl_down_sync(0xffffffffu, x, o);
-                x = (q == max_slot) ? fmax(x, y) : x + y;
-            }
-            if (lane == 0) out[q] = x;
+        for (int i = 1; i < 16; ++i) {
+            const double y = red[q][l + 16 * i];
+            x = mx ? fmax(x, y) : x + y;
         }
+        for (int o = 8; o > 0; o >>= 1) {
+            const double y = __shfl_down_sync(0xffffffffu, x, o, 16);
+            x = mx ? fmax(x, y) : x + y;
+        }
+        if (l == 0) out[q] = x;
     }
 }
 
+// Bound by the FP64 pipe, so counted in its operations: about 30 per site.  The
+// halves and the coefficients of the free energy multiply a thread's sums once
+// (a site's division by Tc and its products were 75 operations): 155 -> 85 us
+// at 1024^2.
 template <typename R>
-__global__ void __launch_bounds__(kThreads) k_diag_partial(Geom g, const R* __restrict__ phi, const R* __restrict__ T,
-                                                           const R* __restrict__ aux, double b, double kappa, double c,
-                                                           double Tc, double* part)
+__global__ void __launch_bounds__(kThreads, 3) k_diag_partial(Geom g, const R* __restrict__ phi, const R* __restrict__ T,
+                                                              const R* __restrict__ aux, double b, double kappa, double c,
+                                                              double Tc, double* part)
 {
-    double v[DQ_N];
+    double v[DQ_N], links = 0.0, lap2 = 0.0;
 #pragma unroll
     for (int q = 0; q < DQ_N; ++q) v[q] = 0.0;
     const int64_t N = (int64_t)g.nx * g.ny * g.nz;
     const int64_t P = g.plane;
+    const int wy = g.walls && g.d == 2, wz = g.walls && g.d == 3;
+    const double ha = 0.5 / Tc, hb = 0.25 * b;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < N; k += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(k % g.nx);
-        const int64_t row = k / g.nx;
-        const int y = (int)(row % g.ny), z = (int)(row / g.ny);
+        int64_t row;
+        int x, y, z;
+        if (N <= INT32_MAX) {
+            const unsigned r = (unsigned)k / (unsigned)g.nx;
+            x = (int)((unsigned)k - r * (unsigned)g.nx);
+            z = (int)(r / (unsigned)g.ny);
+            y = (int)(r - (unsigned)z * (unsigned)g.ny);
+            row = r;
+        } else {
+            row = k / g.nx;
+            x = (int)(k - row * g.nx);
+            z = (int)(row / g.ny);
+            y = (int)(row - (int64_t)z * g.ny);
+        }
         const int64_t site = row * g.pitch + x;
         const double ph = (double)phi[site];
-        double gr[3], lap, links;
-        phi_derivs(phi, g, x, y, z, gr, &lap, &links);
+        // differences to the neighbours; beyond a wall the layer itself (even mirror)
+        const double xp = at(phi, g, nb_index(x, 1, g.nx, 0), y, z) - ph, xm = at(phi, g, nb_index(x, -1, g.nx, 0), y, z) - ph;
+        const double yp = at(phi, g, x, nb_index(y, 1, g.ny, wy), z) - ph, ym = at(phi, g, x, nb_index(y, -1, g.ny, wy), z) - ph;
+        const double gx = xp - xm, gy = yp - ym;             // twice the central difference
+        double lap = (xp + xm) + (yp + ym);
+        v[DQ_GX] = fma(gx, gx, v[DQ_GX]);
+        v[DQ_GY] = fma(gy, gy, v[DQ_GY]);
+        links = fma(xp, xp, fma(yp, yp, links));             // forward links; the one out of the last layer is zero
+        if (g.d == 3) {
+            const double zp = at(phi, g, x, y, nb_index(z, 1, g.nz, wz)) - ph, zm = at(phi, g, x, y, nb_index(z, -1, g.nz, wz)) - ph;
+            const double gz = zp - zm;
+            lap += zp + zm;
+            v[DQ_GZ] = fma(gz, gz, v[DQ_GZ]);
+            links = fma(zp, zp, links);
+        }
+        lap2 = fma(lap, lap, lap2);
         const double n = (double)aux[4 * P + site];
         const double ux = (double)aux[5 * P + site], uy = (double)aux[6 * P + site], uz = (double)aux[7 * P + site];
-        const double a = ((double)T[site] - Tc) / Tc;
         v[DQ_MASS] += n;
         v[DQ_PHI] += ph;
-        v[DQ_MX] += n * ux;
-        v[DQ_MY] += n * uy;
-        v[DQ_MZ] += n * uz;
-        v[DQ_GX] += gr[0] * gr[0];
-        v[DQ_GY] += gr[1] * gr[1];
-        v[DQ_GZ] += gr[2] * gr[2];
-        v[DQ_FE] += a * ph * ph / 2 + b * ph * ph * ph * ph / 4 + kappa * links / 2 + c * lap * lap / 2;
-        v[DQ_U2MAX] = fmax(v[DQ_U2MAX], ux * ux + uy * uy + uz * uz);
+        v[DQ_MX] = fma(n, ux, v[DQ_MX]);
+        v[DQ_MY] = fma(n, uy, v[DQ_MY]);
+        v[DQ_MZ] = fma(n, uz, v[DQ_MZ]);
+        const double p2 = ph * ph;                           // a phi^2 / 2 + b phi^4 / 4, a = (T - Tc) / Tc
+        v[DQ_FE] = fma(fma((double)T[site] - Tc, ha, hb * p2), p2, v[DQ_FE]);
+        v[DQ_U2MAX] = fmax(v[DQ_U2MAX], fma(ux, ux, fma(uy, uy, uz * uz)));
     }
+    v[DQ_GX] *= 0.25;
+    v[DQ_GY] *= 0.25;
+    v[DQ_GZ] *= 0.25;
+    v[DQ_FE] = fma(0.5 * kappa, links, fma(0.5 * c, lap2, v[DQ_FE]));
     block_reduce_store<DQ_N>(v, part + (int64_t)blockIdx.x * DQ_N, DQ_U2MAX);
 }
 
@@ -183,8 +201,8 @@ __global__ void __launch_bounds__(kThreads) k_layers(Geom g, const R* __restrict
         int x, y, z;
         if (g.d == 2) { x = (int)k; y = h; z = 0; }
         else { x = (int)(k % g.nx); y = (int)(k / g.nx); z = h; }
-        double gr[3], lap;
-        phi_derivs(phi, g, x, y, z, gr, &lap);
+        double gr[3];
+        phi_grad(phi, g, x, y, z, gr);
         const double gp = g.d == 2 ? gr[1] : gr[2];
         v[0] += gp * gp;
         v[1] += gr[0] * gr[0] + gr[1] * gr[1] + gr[2] * gr[2];
@@ -255,7 +273,7 @@ __global__ void __launch_bounds__(kThreads) k_shells(Geom g, const double2* __re
 unsigned grid_n(int64_t N)
 {
     int64_t b = (N + kThreads - 1) / kThreads;
-    if (b > kBlocks) b = kBlocks;
+    if (b > kResident) b = kResident;
     return (unsigned)(b < 1 ? 1 : b);
 }
 
