@@ -126,6 +126,8 @@ cudaError_t launch_lb3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cu
 cudaError_t launch_phi3d_compact(const Geom& g, const Phys<double>& p, const StepIO<double>& io, int zc, cudaStream_t s);
 // pass C in FP32 with either stencil, four sites per thread (lf_step3d_phi.cu)
 cudaError_t launch_phi3d_quads(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int zc, cudaStream_t s);
+// FP32: one temperature sub-step, four sites per thread (lf_step3d_phi.cu).
+cudaError_t launch_tsub3d_quads(const Geom& g, const Phys<float>& p, const float* Tin, float* Tout, cudaStream_t s);
 // passes A and C (FP64) of the three-pass step with the isotropic stencils (lf_step3d_iso.cu)
 template <typename R>
 cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& io, cudaStream_t s);

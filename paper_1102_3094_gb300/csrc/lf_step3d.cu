@@ -572,9 +572,13 @@ cudaError_t launch_step3d(const Geom& g, const Phys<R>& p, const StepIO<R>& io, 
 template <typename R>
 cudaError_t launch_tsub3d(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, cudaStream_t s)
 {
-    dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
-    return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub3d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
-                                             : launch_chained(k_tsub3d<R>, grd, blk, 0, s, g, p, Tin, Tout);
+    if constexpr (sizeof(R) == 4) {
+        return launch_tsub3d_quads(g, p, Tin, Tout, s);
+    } else {
+        dim3 blk(32, 8), grd((g.nx + 31) / 32, (g.ny + 7) / 8, g.nz);
+        return g.stencil == LF_STENCIL_ISOTROPIC ? launch_chained(k_tsub3d_iso<R>, grd, blk, 0, s, g, p, Tin, Tout)
+                                                 : launch_chained(k_tsub3d<R>, grd, blk, 0, s, g, p, Tin, Tout);
+    }
 }
 
 template cudaError_t launch_step3d<float>(const Geom&, const Phys<float>&, const StepIO<float>&, bool, cudaStream_t);

@@ -326,6 +326,115 @@ __global__ void __launch_bounds__(128, 3) k_phi3d_iso_q(Geom g, Phys<float> p, S
     if (bad) *reinterpret_cast<volatile int*>(io.flag) = 1;
 }
 
+// One plane of T around a thread's four sites: the sites, the sums of their
+// four in-plane neighbours and (isotropic) of their four diagonal ones, in the
+// order of k_tsub3d / k_tsub3d_iso.
+struct TPlane {
+    Q4 c, cross, diag;
+};
+
+// A temperature sub-step (k_tsub3d, k_tsub3d_iso) with four sites per thread
+// marching along z, so that each plane's in-plane sums are formed once for the
+// three planes that use them and loads are 16 bytes.  Bound by memory on large
+// lattices (384^3: 453 MB, 67 us) and by the launch on small ones.  One site per
+// thread took 19 (7) loads of 4 bytes per site: isotropic 384^3 335 -> 95 us,
+// 250 x 243 x 190 72.7 -> 23.7, 32 x 32 x 256 3.25 -> 2.4; compact 384^3 229 -> 77.
+// Every site goes through the scalar kernels' operations in their order (the
+// same bits); a plane beyond a wall is 2 T_w minus the wall plane.
+template <int LX, bool ISO>
+__global__ void __launch_bounds__(128) k_tsub3d_q(Geom g, Phys<float> p, const float* __restrict__ Tin,
+                                                  float* __restrict__ Tout, int zc)
+{
+    const Quad<LX> q(g);
+    const int za = blockIdx.z * zc, zb = min(za + zc, g.nz);
+    const int nz = g.nz, pitch = g.pitch, walls = g.walls;
+    const int zs = g.ny * pitch;                 // 32-bit offsets: Q * padded sites < 2^31 (checked at creation)
+    const int row = q.y * pitch;
+    const int rl = (q.y == 0 ? g.ny - 1 : q.y - 1) * pitch, rr = (q.y + 1 == g.ny ? 0 : q.y + 1) * pitch;
+    const float tw2 = 2.f * p.T_w;
+    chain_wait();
+    // plane z; with `image`, also what the plane beyond a wall at z is to it
+    auto plane = [&](int z, TPlane* image) {
+        const float* f = Tin + z * zs;
+        TPlane t;
+        t.c = q.load(f + row);
+        const Q4 l4 = q.load(f + rl), r4 = q.load(f + rr);
+        const Row c = q.around(t.c, q.beside(f + row));
+        Row l{}, r{};
+        if constexpr (ISO) {
+            l = q.around(l4, q.beside(f + rl));
+            r = q.around(r4, q.beside(f + rr));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            t.cross.v[i] = c.e[i] + c.e[i + 2] + l4.v[i] + r4.v[i];
+            t.diag.v[i] = ISO ? l.e[i] + l.e[i + 2] + r.e[i] + r.e[i + 2] : 0.f;
+        }
+        if (image) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                image->c.v[i] = tw2 - t.c.v[i];
+                image->cross.v[i] = ISO ? (tw2 - c.e[i]) + (tw2 - c.e[i + 2]) + (tw2 - l4.v[i]) + (tw2 - r4.v[i]) : 0.f;
+                image->diag.v[i] = 0.f;          // never used beyond a wall
+            }
+        }
+        return t;
+    };
+    TPlane dn{}, mid, up{}, beyond{};
+    const bool lo = walls && za == 0;
+    if (!lo) dn = plane(za == 0 ? nz - 1 : za - 1, nullptr);
+    mid = plane(za, lo ? &dn : nullptr);
+    if (walls && za == nz - 1) plane(za, &beyond);   // the segment starts at the last plane
+    for (int z = za; z < zb; ++z) {
+        const bool hi = walls && z == nz - 1;
+        if (hi) {
+            up = beyond;
+        } else {
+            const int zu = z + 1 == nz ? 0 : z + 1;
+            if (z + 2 < nz) asm volatile("prefetch.global.L2 [%0];" ::"l"(Tin + (z + 2) * zs + row + q.x));
+            up = plane(zu, walls && zu == nz - 1 ? &beyond : nullptr);
+        }
+        const bool held = walls && g.t_mode == LF_TWALL_LAYERS && (z == 0 || z == nz - 1);
+        Q4 o;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float t0 = mid.c.v[i];
+            float lap;
+            if constexpr (ISO) {
+                const float nn = mid.cross.v[i] + dn.c.v[i] + up.c.v[i];
+                const float ed = mid.diag.v[i] + dn.cross.v[i] + up.cross.v[i];
+                lap = fmaf(-24.f, t0, fmaf(2.f, nn, ed)) * (1.f / 6.f);
+            } else {
+                lap = fmaf(-6.f, t0, mid.cross.v[i] + up.c.v[i] + dn.c.v[i]);
+            }
+            o.v[i] = held ? p.T_w : fmaf(p.dxi, lap, t0);
+        }
+        if (q.act) q.store(Tout + z * zs + row, o);
+        dn = mid;
+        mid = up;
+    }
+    chain_next();
+}
+
+// Lanes per row for a row of nq quads: the widest of 32, 16, 8 that leaves the
+// fewest lanes past the end of a row.
+int quad_lanes(int nq)
+{
+    int lx = 32;
+    for (int c = 16; c >= 8; c /= 2)
+        if ((nq + c - 1) / c * c < (nq + lx - 1) / lx * lx) lx = c;
+    return lx;
+}
+
+template <int LX>
+cudaError_t launch_tsub_q(const Geom& g, const Phys<float>& p, const float* Tin, float* Tout, int zc, cudaStream_t s)
+{
+    constexpr int NT = 128, RY = NT / LX;
+    const dim3 grid(((g.nx + 3) / 4 + LX - 1) / LX, (g.ny + RY - 1) / RY, (g.nz + zc - 1) / zc);
+    return launch_chained(g.stencil == LF_STENCIL_ISOTROPIC ? k_tsub3d_q<LX, true> : k_tsub3d_q<LX, false>, grid, NT, 0, s, g,
+                          p, Tin, Tout, zc);
+}
+
 template <int LX>
 cudaError_t launch_q(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int zc, cudaStream_t s)
 {
@@ -340,11 +449,7 @@ cudaError_t launch_q(const Geom& g, const Phys<float>& p, const StepIO<float>& i
 
 cudaError_t launch_phi3d_quads(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int zc, cudaStream_t s)
 {
-    // lanes per row: the widest of 32, 16, 8 that leaves the fewest lanes past the end of a row
-    const int nq = (g.nx + 3) / 4;
-    int lx = 32;
-    for (int c = 16; c >= 8; c /= 2)
-        if ((nq + c - 1) / c * c < (nq + lx - 1) / lx * lx) lx = c;
+    const int nq = (g.nx + 3) / 4, lx = quad_lanes(nq);
     if (zc <= 0) {
         // Planes per segment: the more the fewer planes are read twice, as long
         // as every SM has its fill of blocks (six compact, three isotropic, of
@@ -362,6 +467,27 @@ cudaError_t launch_phi3d_quads(const Geom& g, const Phys<float>& p, const StepIO
         }
     }
     return lx == 32 ? launch_q<32>(g, p, io, zc, s) : lx == 16 ? launch_q<16>(g, p, io, zc, s) : launch_q<8>(g, p, io, zc, s);
+}
+
+cudaError_t launch_tsub3d_quads(const Geom& g, const Phys<float>& p, const float* Tin, float* Tout, cudaStream_t s)
+{
+    int sms = 0;
+    const cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const int nq = (g.nx + 3) / 4, lx = quad_lanes(nq), ry = 128 / lx;
+    const int64_t cols = (int64_t)((nq + lx - 1) / lx) * ((g.ny + ry - 1) / ry);
+    // Planes per segment: with 8 to 32 large lattices differ by 5 %; small ones
+    // take the shortest segments (32 x 32 x 256: 2.4 us with 2 planes, 4.1 with
+    // 8), and four blocks per SM hide the loads' latency (128^3 isotropic: 6.0 us
+    // with 6 planes, 7.2 with 2, 7.4 with 12).
+    int zc = 2;
+    for (int c : {12, 8, 6, 4, 3, 2}) {
+        zc = c;
+        if (cols * ((g.nz + c - 1) / c) >= 4 * (int64_t)sms) break;
+    }
+    return lx == 32   ? launch_tsub_q<32>(g, p, Tin, Tout, zc, s)
+           : lx == 16 ? launch_tsub_q<16>(g, p, Tin, Tout, zc, s)
+                      : launch_tsub_q<8>(g, p, Tin, Tout, zc, s);
 }
 
 }  // namespace lf
