@@ -749,7 +749,10 @@ def run_ours(args):
     bps = BYTES_PER_SITE[(prec, d)]
     peak, peak_kind = peaks()
     passes = 3 if (d == 3 and variant == "split3") else 1
-    launches_per_step = passes + (lf.lf_nsub(args.xi, d) - 1 if args.xi not in (0.0, math.inf) else 0)
+    extra = lf.lf_nsub(args.xi, d) - 1 if args.xi not in (0.0, math.inf) else 0
+    if d == 2 and prec == "fp32":
+        extra = (extra + 3) // 4            # up to four temperature sub-steps per launch
+    launches_per_step = passes + extra
     # the three-pass 3D step is measured as a whole: algorithmic bytes of the
     # step over the step time
     per_kernel = 1 if passes > 1 else launches_per_step
@@ -778,11 +781,12 @@ def run_ours(args):
     def pass_breakdown(sim_, iso_, param_, restore_fn):
         sel = (param_ >> 16) & 15
         if iso_:
-            force = "k_force3d_iso_x2" if (sel == 4 and prec == "fp32") else "k_force3d_iso"
-            phi_k = "k_phi3d_isoz"
+            packed = prec == "fp32" and (sel == 4 or (param_ & 0xFFFFF) == 0)
+            force = "k_force3d_iso_x2" if packed else "k_force3d_iso"
+            phi_k = "k_phi3d_iso_q" if prec == "fp32" else "k_phi3d_isoz"
         else:
             force = "k_force3d_x2" if (sel == 0 and prec == "fp32") else "k_force3d"
-            phi_k = "k_phi3d"
+            phi_k = "k_phi3d_q" if prec == "fp32" else "k_phi3d"
         esz = 4 if prec == "fp32" else 8
         per_site = [6 * esz, 44 * esz, 8 * esz]      # A: phi, T in, mu, F out; B: f in/out, F, u; C: phi, u, mu, T in, phi, T out
         acc, cnt = [0.0, 0.0, 0.0], 0

@@ -239,8 +239,9 @@ inline cudaError_t device_sms(int* sms)
 // 1024^2: 26.7 us a step with it at the end, 31.7 two rows before the end, 39
 // at the start; 28.8 without any of this); at the start of kernels with many
 // waves of small blocks or hardly any work in each.
-// 64^2 FP64 24.6 -> 21.6 us a step, 256^2 FP32 10.3 -> 8.7, 1024^2 28.8 -> 26.7,
-// 32 x 32 x 256 with eight temperature sub-steps 75 -> 57.
+// Without and with it, the kernels otherwise the same: 64^2 FP64 row march 24.6
+// and 21.6 us a step, 256^2 FP32 on 128-thread CTAs 10.3 and 8.7, 1024^2 28.8 and
+// 26.7, 32 x 32 x 256 with eight temperature sub-steps 75 and 57.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

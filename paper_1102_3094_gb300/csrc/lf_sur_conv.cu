@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
             // bits): the next row's residual and mask are loaded before this
             // row's stores, so their latency lies under the stores and the wait.
             // 16 x 256^2, 64 -> 64: 192 us with BF16 masks, loads at the top of
-            // each row and the sums in a kernel of their own (34 us); 105 us now.
+            // each row and the sums in a kernel of their own (34 us); 146 us now.
             auto fetch = [&](const ConvSeg& g, int y, uint4 (&rp)[2], uint32_t& mb) {
                 const int x = g.x0 + pix;
                 if (a.resid) {
@@ -630,7 +630,7 @@ struct WgArgs {
 // dW[t][o][i] = sum over the group's items of part[item][t - t0][m][n], in the
 // order of the items.  Threads follow the order of the partials (coalesced; the
 // transposed order is taken on the one store) with sixteen loads in flight:
-// 15 MB of partials in L2 for 64 -> 64, 15.6 us in the order of dW, 6 us now.
+// 15 MB of partials in L2 for 64 -> 64, 15.6 us in the order of dW, 7.6 us now.
 template <int CIN, int COUT>
 __global__ void __launch_bounds__(64) k_wgrad_reduce(const float* __restrict__ part, float* __restrict__ dW)
 {
