@@ -426,24 +426,27 @@ void default_rows(lf_ens* e)
     const float lag[2] = {5.5f, 10.f};
     for (int iso = 0; iso < 2; ++iso) {
         std::vector<int> members;
+        std::map<std::pair<int, int>, int> sizes;                        // (nx, ny): runs
         int tallest = 0;
         for (int r = 0; r < e->nruns; ++r) {
             const Geom& g = e->runs[r]->g;
             if ((g.stencil == LF_STENCIL_ISOTROPIC) != (iso == 1)) continue;
             members.push_back(r);
+            ++sizes[{g.nx, g.ny}];
             tallest = std::max(tallest, g.ny);
         }
         if (members.empty()) continue;
         int best = 1;
         float best_us = -1.f;
-        std::vector<std::pair<int, int64_t>> lanes(members.size());      // rows per lane, items
+        std::vector<std::pair<int, int64_t>> lanes;                      // rows per lane, items
         for (int h = 1; h <= std::max(1, tallest / 2) && h <= 512; ++h) {
             int64_t items = 0;
-            for (size_t m = 0; m < members.size(); ++m) {
-                const Geom& g = e->runs[members[m]]->g;
-                const int np = pairs_for(g.ny, h);
-                lanes[m] = {(g.ny + 2 * np - 1) / (2 * np), (int64_t)np * ((g.nx + MarchCfg<64>::U - 1) / MarchCfg<64>::U)};
-                items += lanes[m].second;
+            lanes.clear();
+            for (const auto& [size, runs] : sizes) {
+                const auto [nx, ny] = size;
+                const int64_t np = pairs_for(ny, h), strips = (nx + MarchCfg<64>::U - 1) / MarchCfg<64>::U;
+                lanes.push_back({(int)((ny + 2 * np - 1) / (2 * np)), np * strips * runs});
+                items += lanes.back().second;
             }
             std::sort(lanes.begin(), lanes.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
             const int64_t B = std::min<int64_t>(items, 6 * (int64_t)sms);
