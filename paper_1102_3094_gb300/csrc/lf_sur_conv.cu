@@ -101,6 +101,30 @@ __device__ __forceinline__ ConvSeg conv_segment(int64_t q, int64_t r1, int NY, i
     return g;
 }
 
+// 16 channels of a pixel, 32 bytes: in one access (a whole sector; a thread's
+// neighbours are 128 bytes away, so two of 16 bytes touch every line twice) when
+// the buffers allow it.  16 x 256^2: backward 64 -> 64 146 -> 113 us, 16 -> 64 113
+// -> 75, forward 16 -> 64 89 -> 68 (64 -> 64, whose residual comes from the ring,
+// 100 either way).
+__device__ __forceinline__ void put16(__nv_bfloat16* d, const uint4* h, int sectors)
+{
+    if (sectors) {
+        tc::st_global_32(d, h[0], h[1]);
+    } else {
+        reinterpret_cast<uint4*>(d)[0] = h[0];
+        reinterpret_cast<uint4*>(d)[1] = h[1];
+    }
+}
+__device__ __forceinline__ void get16(const __nv_bfloat16* s, uint4 (&h)[2], int sectors)
+{
+    if (sectors) {
+        tc::ld_global_32(s, h[0], h[1]);
+    } else {
+        h[0] = reinterpret_cast<const uint4*>(s)[0];
+        h[1] = reinterpret_cast<const uint4*>(s)[1];
+    }
+}
+
 template <int CIN, int COUT, bool BWD>
 __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
     k_conv3x3(const __grid_constant__ CUtensorMap tin, const __grid_constant__ CUtensorMap tw, ConvArgs a)
@@ -307,13 +331,12 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
             // bits): the next row's residual and mask are loaded before this
             // row's stores, so their latency lies under the stores and the wait.
             // 16 x 256^2, 64 -> 64: 192 us with BF16 masks, loads at the top of
-            // each row and the sums in a kernel of their own (34 us); 146 us now.
+            // each row and the sums in a kernel of their own (34 us); 146 us
+            // without these, 113 us with 32-byte accesses.
             auto fetch = [&](const ConvSeg& g, int y, uint4 (&rp)[2], uint32_t& mb) {
                 const int x = g.x0 + pix;
                 if (a.resid) {
-                    const uint4* rs = reinterpret_cast<const uint4*>(a.resid + pix_off(g.b, y, x, NY, NX) * COUT + c0);
-                    rp[0] = rs[0];
-                    rp[1] = rs[1];
+                    get16(a.resid + pix_off(g.b, y, x, NY, NX) * COUT + c0, rp, a.sectors);
                 }
                 mb = a.mbits[(((int64_t)g.b * NY + y) * 4 + part) * NX + x];
             };
@@ -375,14 +398,8 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
                     }
                     auto store = [&](__nv_bfloat16* base, const __nv_bfloat16* h) {
                         const uint4* hv = reinterpret_cast<const uint4*>(h);
-                        uint4* d = reinterpret_cast<uint4*>(base + po * COUT + c0);
-                        d[0] = hv[0];
-                        d[1] = hv[1];
-                        if (halo_hi || halo_lo) {
-                            uint4* dh = reinterpret_cast<uint4*>(base + po_h * COUT + c0);
-                            dh[0] = hv[0];
-                            dh[1] = hv[1];
-                        }
+                        put16(base + po * COUT + c0, hv, a.sectors);
+                        if (halo_hi || halo_lo) put16(base + po_h * COUT + c0, hv, a.sectors);
                     };
                     if (a.out) store(a.out, ho);
                     store(a.out2, hm);
@@ -414,9 +431,7 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
                 // residual and mask loads issued before the wait for the row's MMAs
                 uint4 rp[2] = {}, mp[2] = {};
                 if (a.resid && !ring_res) {
-                    const uint4* rs = reinterpret_cast<const uint4*>(a.resid + po * COUT + c0);
-                    rp[0] = rs[0];
-                    rp[1] = rs[1];
+                    get16(a.resid + po * COUT + c0, rp, a.sectors);
                 }
                 if (a.mask) {
                     const uint4* ms = reinterpret_cast<const uint4*>(a.mask + po * COUT + c0);
@@ -499,14 +514,8 @@ __global__ void __launch_bounds__(conv_threads<COUT>(), 1)
                 auto store = [&](__nv_bfloat16* base, const __nv_bfloat16* h) {
                     if (!base) return;
                     const uint4* hv = reinterpret_cast<const uint4*>(h);
-                    uint4* d = reinterpret_cast<uint4*>(base + po * COUT + c0);
-                    d[0] = hv[0];
-                    d[1] = hv[1];
-                    if (halo_hi || halo_lo) {
-                        uint4* dh = reinterpret_cast<uint4*>(base + po_h * COUT + c0);
-                        dh[0] = hv[0];
-                        dh[1] = hv[1];
-                    }
+                    put16(base + po * COUT + c0, hv, a.sectors);
+                    if (halo_hi || halo_lo) put16(base + po_h * COUT + c0, hv, a.sectors);
                 };
                 store(a.zout, hz);
                 store(a.out, ho);
@@ -583,8 +592,11 @@ cudaError_t launch_conv(const ConvArgs& a, cudaStream_t s)
     return launch_chained(k_conv3x3<CIN, COUT, BWD>, blocks, conv_threads<COUT>(), S::BYTES, s, m, mw, a);
 }
 
-cudaError_t conv3x3(int cin, int cout, const ConvArgs& a, cudaStream_t s)
+cudaError_t conv3x3(int cin, int cout, const ConvArgs& args, cudaStream_t s)
 {
+    ConvArgs a = args;
+    const uintptr_t bits = (uintptr_t)a.out | (uintptr_t)a.out2 | (uintptr_t)a.zout | (uintptr_t)a.resid;
+    a.sectors = bits % 32 == 0;                  // a pixel's channels are a multiple of 32 bytes
     if (a.mbits) {
         if (cin == 16 && cout == 64) return launch_conv<16, 64, true>(a, s);
         if (cin == 64 && cout == 64) return launch_conv<64, 64, true>(a, s);

@@ -35,6 +35,7 @@ struct ConvArgs {
     // was itself started after they were written), so they may be read before
     // that kernel has finished
     int old_weights;
+    int sectors;                 // set by conv3x3: out, out2, zout and resid are 32-byte aligned
 };
 
 // `mbits` selects the backward form: acc (+ resid) -> out (may be null) and out2 = out where the bit is set.

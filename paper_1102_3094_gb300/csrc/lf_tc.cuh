@@ -198,6 +198,21 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, int c0,
                  : "memory");
 }
 
+// 32 bytes (a whole sector) in one access; p is 32-byte aligned.
+__device__ __forceinline__ void st_global_32(void* p, uint4 a, uint4 b)
+{
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x), "r"(a.y), "r"(a.z),
+                 "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void ld_global_32(const void* p, uint4& a, uint4& b)
+{
+    asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(p)
+                 : "memory");
+}
+
 // 16 consecutive FP32 columns of this thread's TMEM lane (32x32b shape: warp
 // w of a warpgroup reads lanes 32w .. 32w + 31).
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
