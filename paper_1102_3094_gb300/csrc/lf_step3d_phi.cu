@@ -342,8 +342,7 @@ struct TPlane {
 // Every site goes through the scalar kernels' operations in their order (the
 // same bits); a plane beyond a wall is 2 T_w minus the wall plane.
 template <int LX, bool ISO>
-__global__ void __launch_bounds__(128) k_tsub3d_q(Geom g, Phys<float> p, const float* __restrict__ Tin,
-                                                  float* __restrict__ Tout, int zc)
+__global__ void __launch_bounds__(128) k_tsub3d_q(Geom g, Phys<float> p, const float* Tin, float* Tout, int zc)
 {
     const Quad<LX> q(g);
     const int za = blockIdx.z * zc, zb = min(za + zc, g.nz);
