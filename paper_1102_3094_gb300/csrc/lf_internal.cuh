@@ -229,9 +229,9 @@ inline cudaError_t device_sms(int* sms)
 // calls chain_wait() before it touches memory that another kernel writes,
 // which waits until every earlier grid has finished and its writes are
 // visible.  Everything after that is ordered as in a plain launch, also when
-// the predecessor is a kernel or copy that knows nothing of this.  (A pointer
-// to such memory is not declared __restrict__ in the kernel's parameters: the
-// compiler may load through those ahead of the wait.)
+// the predecessor is a kernel or copy that knows nothing of this.  (No pointer
+// to such memory is declared __restrict__, among the kernel's parameters or
+// inside it: the compiler may load through those ahead of the wait.)
 //
 // Where chain_next() stands: at the end of the kernels whose blocks fill the
 // SMs once or twice, because blocks of the successor that come in earlier take

@@ -322,8 +322,7 @@ __device__ __forceinline__ void march2d_segment(const Geom& g, const Phys<R>& p,
 // One explicit temperature sub-step at site (x, y): T += dxi nabla^2 T with
 // the wall rule of the context (layers held at T_w, or a halfway ghost).
 template <typename R>
-__device__ __forceinline__ void tsub2d_site(const Geom& g, const Phys<R>& p, const R* __restrict__ Tin,
-                                            R* __restrict__ Tout, int x, int y)
+__device__ __forceinline__ void tsub2d_site(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, int x, int y)
 {
     const int nx = g.nx, ny = g.ny, pitch = g.pitch;
     const int site = y * pitch + x;

@@ -516,12 +516,12 @@ __global__ void __launch_bounds__(256) k_phi3d_isoz(Geom g, Phys<R> p, StepIO<R>
     const int64_t zs = (int64_t)ny * pitch;
     const bool hyd = p.hydro != 0;
     const bool halfway = walls && g.t_mode == LF_TWALL_HALFWAY;
-    const R* __restrict__ mu = io.mu;
-    const R* __restrict__ ph = io.phi_in;
-    const R* __restrict__ T = io.T_in;
-    const R* __restrict__ ux = io.u[0];
-    const R* __restrict__ uy = io.u[1];
-    const R* __restrict__ uz = io.u[2];
+    const R* mu = io.mu;
+    const R* ph = io.phi_in;
+    const R* T = io.T_in;
+    const R* ux = io.u[0];
+    const R* uy = io.u[1];
+    const R* uz = io.u[2];
     auto zmap = [&](int zl) -> int64_t {
         int z = zl;
         if (walls) z = z < 0 ? 0 : (z >= nz ? nz - 1 : z);

@@ -489,14 +489,14 @@ __global__ void __launch_bounds__(256) k_phi3d(Geom g, Phys<R> p, StepIO<R> io, 
     const int xl = x == 0 ? nx - 1 : x - 1, xr = x + 1 == nx ? 0 : x + 1;
     const int64_t ryl = (int64_t)(y == 0 ? ny - 1 : y - 1) * pitch, ryr = (int64_t)(y + 1 == ny ? 0 : y + 1) * pitch;
     const R half = R(0.5);
-    const R* __restrict__ mu = io.mu;
-    const R* __restrict__ ph = io.phi_in;
-    const R* __restrict__ T = io.T_in;
-    const R* __restrict__ ux = io.u[0];
-    const R* __restrict__ uy = io.u[1];
-    const R* __restrict__ uz = io.u[2];
-    R* __restrict__ phi_out = io.phi_out;
-    R* __restrict__ T_out = io.T_out;
+    const R* mu = io.mu;
+    const R* ph = io.phi_in;
+    const R* T = io.T_in;
+    const R* ux = io.u[0];
+    const R* uy = io.u[1];
+    const R* uz = io.u[2];
+    R* phi_out = io.phi_out;
+    R* T_out = io.T_out;
     // plane index of the neighbour below / above: wrap (periodic) or the plane itself (walls)
     auto below = [&](int z) { return z == 0 ? (walls ? 0 : nz - 1) : z - 1; };
     auto above = [&](int z) { return z + 1 == nz ? (walls ? z : 0) : z + 1; };

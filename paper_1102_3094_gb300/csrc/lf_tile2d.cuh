@@ -307,8 +307,7 @@ __device__ __forceinline__ void step2d_tile(const Geom& g, const Phys<R>& p, con
 // holds 2 T_w - T of the site's own row (halfway ghost); with held wall
 // layers the interior never reaches past them.
 template <typename R>
-__device__ __forceinline__ void tsub2d_site_iso(const Geom& g, const Phys<R>& p, const R* __restrict__ Tin,
-                                                R* __restrict__ Tout, int x, int y)
+__device__ __forceinline__ void tsub2d_site_iso(const Geom& g, const Phys<R>& p, const R* Tin, R* Tout, int x, int y)
 {
     const int nx = g.nx, ny = g.ny, pitch = g.pitch;
     const int site = y * pitch + x;

@@ -31,6 +31,10 @@ def matching(text, i):
     raise AssertionError("unbalanced")
 
 
+def files():
+    return sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))
+
+
 def kernels(text):
     """(name, parameters, body) of every kernel defined in `text`."""
     for m in re.finditer(r"__global__", text):
@@ -46,7 +50,7 @@ def kernels(text):
 
 def chained():
     out = []
-    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh"))):
+    for path in files():
         out += [(os.path.basename(path), *k) for k in kernels(source(path)) if "chain_wait()" in k[2]]
     return out                                   # (file, name, parameters, body)
 
@@ -60,3 +64,12 @@ def test_the_scan_finds_the_kernels():
 @pytest.mark.parametrize("kernel", chained(), ids=lambda k: k[1])
 def test_no_restrict_parameter_for_memory_of_the_predecessor(kernel):
     assert "__restrict__" not in HOST_TABLES.sub("", kernel[2])
+
+
+@pytest.mark.parametrize("path", files(), ids=os.path.basename)
+def test_no_restrict_outside_kernel_parameters(path):
+    """Nor on a pointer made inside a kernel or a function that kernels share."""
+    text = source(path)
+    for _, params, _ in kernels(text):
+        text = text.replace(params, "")
+    assert "__restrict__" not in text
