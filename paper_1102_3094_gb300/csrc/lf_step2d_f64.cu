@@ -107,7 +107,9 @@ __global__ void __launch_bounds__(NT) k_step2d_f64(Geom g, Phys<double> p, StepI
 
     const int nx = g.nx, ny = g.ny, pitch = g.pitch, walls = g.walls;
     const int plane = (int)g.plane;                          // 32-bit offsets: Q * padded sites < 2^31
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
+    const unsigned across = (unsigned)(nx + TX - 1) / TX;    // tiles per row of them
+    const int ty = (int)(blockIdx.x / across), tx = (int)(blockIdx.x - ty * across);
+    const int x0 = tx * TX, y0 = ty * TY;
     bool bad = false;
 
     chain_wait();
@@ -326,7 +328,8 @@ cudaError_t launch_tile(const Geom& g, const Phys<double>& p, const StepIO<doubl
     static unsigned long long attr_done[2] = {};             // per instantiation and device
     const cudaError_t e = raise_smem_limit(kern, (int)bytes, &attr_done[iso]);
     if (e != cudaSuccess) return e;
-    const dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY);
+    // all tiles on x: a narrow lattice may have more rows of them than the 65,535 that y takes
+    const dim3 grid((unsigned)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY));
     return launch_chained(kern, grid, NT, bytes, s, g, p, io);
 }
 
