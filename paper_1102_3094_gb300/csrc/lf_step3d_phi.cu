@@ -51,8 +51,10 @@ struct Quad {
     __device__ Quad(const Geom& g)
     {
         const int lane = threadIdx.x % LX;
-        const int nq = (g.nx + 3) / 4, q = blockIdx.x * LX + lane;
-        y = blockIdx.y * (blockDim.x / LX) + threadIdx.x / LX;
+        const int nq = (g.nx + 3) / 4;
+        const unsigned across = (unsigned)(nq + LX - 1) / LX, by = blockIdx.x / across;   // blocks per row of them
+        const int q = (int)(blockIdx.x - by * across) * LX + lane;
+        y = (int)(by * (blockDim.x / LX)) + threadIdx.x / LX;
         act = q < nq && y < g.ny;
         if (y >= g.ny) y = g.ny - 1;
         x = q < nq ? 4 * q : 0;
@@ -425,11 +427,20 @@ int quad_lanes(int nq)
     return lx;
 }
 
+// `nt` threads take nt / LX rows over `zc` planes.  The blocks of all rows are on
+// x: y takes 65,535, which a long lattice exceeds.
+template <int LX>
+dim3 quad_grid(const Geom& g, int nt, int zc)
+{
+    const int ry = nt / LX;
+    return dim3((unsigned)(((g.nx + 3) / 4 + LX - 1) / LX) * ((g.ny + ry - 1) / ry), 1, (g.nz + zc - 1) / zc);
+}
+
 template <int LX>
 cudaError_t launch_tsub_q(const Geom& g, const Phys<float>& p, const float* Tin, float* Tout, int zc, cudaStream_t s)
 {
-    constexpr int NT = 128, RY = NT / LX;
-    const dim3 grid(((g.nx + 3) / 4 + LX - 1) / LX, (g.ny + RY - 1) / RY, (g.nz + zc - 1) / zc);
+    constexpr int NT = 128;
+    const dim3 grid = quad_grid<LX>(g, NT, zc);
     return launch_chained(g.stencil == LF_STENCIL_ISOTROPIC ? k_tsub3d_q<LX, true> : k_tsub3d_q<LX, false>, grid, NT, 0, s, g,
                           p, Tin, Tout, zc);
 }
@@ -437,8 +448,8 @@ cudaError_t launch_tsub_q(const Geom& g, const Phys<float>& p, const float* Tin,
 template <int LX>
 cudaError_t launch_q(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int zc, cudaStream_t s)
 {
-    constexpr int NT = 128, RY = NT / LX;
-    const dim3 grid(((g.nx + 3) / 4 + LX - 1) / LX, (g.ny + RY - 1) / RY, (g.nz + zc - 1) / zc);
+    constexpr int NT = 128;
+    const dim3 grid = quad_grid<LX>(g, NT, zc);
     if (g.stencil == LF_STENCIL_ISOTROPIC)
         return launch_chained(p.hydro ? k_phi3d_iso_q<LX, true> : k_phi3d_iso_q<LX, false>, grid, NT, 0, s, g, p, io, zc);
     return launch_chained(p.hydro ? k_phi3d_q<LX, true> : k_phi3d_q<LX, false>, grid, NT, 0, s, g, p, io, zc);

@@ -16,7 +16,7 @@ def one_step(period, times, **kw):
     torch.manual_seed(5)
     out = []
     for n in (times, 1):
-        sim = lf.Lattice(ny=period * n, walls=0, xi=0.1, **kw)
+        sim = lf.Lattice(ny=period * n, walls=0, **dict(dict(xi=0.1), **kw))
         shape = (sim.shape[:-2] + (1, period, sim.shape[-1]))
         dt = torch.float64 if kw["precision"] == "fp64" else torch.float32
         if n == times:
@@ -36,3 +36,19 @@ def test_fp64_2d(nx, stencil):
     long, short = one_step(16, 16384, nx=nx, precision="fp64", stencil=stencil)
     for a, b in zip(long, short):
         assert (a - b).abs().max() <= 200 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("stencil", ["compact", "isotropic"])
+def test_fp32_3d_quads(stencil):
+    # 262,144 rows of 25 quads, 32 lanes each: 65,536 blocks of four rows; xi = 0.1 is one sub-step, so T
+    # takes the phi pass.  Rows do the same operations wherever they lie.
+    long, short = one_step(16, 16384, d=3, nx=100, nz=2, precision="fp32", stencil=stencil, hydro=0)
+    for a, b in zip(long, short):
+        assert (a - b).abs().max() == 0
+
+
+@pytest.mark.parametrize("stencil", ["compact", "isotropic"])
+def test_fp32_3d_sub_steps(stencil):
+    long, short = one_step(16, 16384, d=3, nx=100, nz=2, precision="fp32", stencil=stencil, hydro=0, xi=0.3)
+    for a, b in zip(long, short):
+        assert (a - b).abs().max() == 0
