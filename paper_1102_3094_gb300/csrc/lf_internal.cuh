@@ -238,7 +238,10 @@ inline cudaError_t device_sms(int* sms)
 // the places that happen to be free and then run unevenly spread (2D march at
 // 1024^2: 26.7 us a step with it at the end, 31.7 two rows before the end, 39
 // at the start; 28.8 without any of this); at the start of kernels with many
-// waves of small blocks or hardly any work in each.
+// waves of small blocks or hardly any work in each.  FP64 kernels whose successor
+// has large blocks leave it out, which puts it at their end: a block that is
+// badly placed waits for its SM's FP64 pipe (3D collision and sub-steps at 32 x
+// 32 x 256: isotropic step 660 -> 517 us, compact with eight sub-steps 525 -> 366).
 // Without and with it, the kernels otherwise the same: 64^2 FP64 row march 24.6
 // and 21.6 us a step, 256^2 FP32 on 128-thread CTAs 10.3 and 8.7, 1024^2 28.8 and
 // 26.7, 32 x 32 x 256 with eight temperature sub-steps 75 and 57.

@@ -132,8 +132,10 @@ __global__ void __launch_bounds__(NT) k_step2d_f64(Geom g, Phys<double> p, StepI
     //   iso = phi^2 (a / 2 + 3/4 b phi^2) - kappa (phi psi + |grad phi|^2 / 2)
     //       + c (phi lam + psi^2 / 2 + grad phi . grad psi)
     //   P_ab = iso delta_ab + kappa d_a d_b - c (d_a s_b + d_b s_a)
+    // with a = (T - Tc) / Tc from the difference, which is exact near Tc (a fused
+    // T / (2 Tc) - 1/2 has the rounding of 1 / Tc instead: 2e-17 at T = Tc)
     {
-        const double ah = 0.5 * p.inv_Tc, a0 = -0.5 * p.Tc * p.inv_Tc, b34 = 0.75 * p.b;
+        const double b34 = 0.75 * p.b;
         const double kL = -p.kappa / D::KL, cL = p.c / (D::KL * D::KL);
         const double g2 = 0.5 / (D::KD * D::KD), p2 = 0.5 / (D::KL * D::KL), gs = 1.0 / (D::KD * D::KD * D::KL);
         const double kD = p.kappa / (D::KD * D::KD), cD = -p.c * gs;
@@ -142,13 +144,13 @@ __global__ void __launch_bounds__(NT) k_step2d_f64(Geom g, Phys<double> p, StepI
             const int cp = (ly + 2) * W4 + lx + 2, cs = (ly + 1) * W3 + lx + 1;
             const double ph = sphi[cp], ps = spsi[cs];
             const double lam = D::template lap<W3>(spsi, cs);
-            const double ha = fma(ah, sT[k], a0), ph2 = ph * ph;              // a / 2
-            smu[k] = fma(cL, lam, fma(kL, ps, ph * fma(p.b, ph2, ha + ha)));
+            const double a = (sT[k] - p.Tc) * p.inv_Tc, ph2 = ph * ph;
+            smu[k] = fma(cL, lam, fma(kL, ps, ph * fma(p.b, ph2, a)));
             if (p.hydro) {
                 const double dx = D::template dx<W4>(sphi, cp), dy = D::template dy<W4>(sphi, cp);
                 const double ex = D::template dx<W3>(spsi, cs), ey = D::template dy<W3>(spsi, cs);
                 const double xx = dx * dx, yy = dy * dy, ux = dx * ex, uy = dy * ey;
-                double iso = ph2 * fma(b34, ph2, ha);
+                double iso = ph2 * fma(b34, ph2, 0.5 * a);
                 iso = fma(-p.kappa, fma(g2, xx + yy, ph * ps * (1.0 / D::KL)), iso);
                 iso = fma(p.c, fma(gs, ux + uy, fma(p2 * ps, ps, ph * lam * (1.0 / (D::KL * D::KL)))), iso);
                 sPxx[k] = fma(kD, xx, fma(2.0 * cD, ux, iso));

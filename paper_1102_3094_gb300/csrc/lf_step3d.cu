@@ -485,7 +485,6 @@ __global__ void k_tsub3d(Geom g, Phys<R> p, const R* Tin, R* Tout)
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
-    chain_next();
     chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch;
@@ -520,7 +519,6 @@ __global__ void k_tsub3d_iso(Geom g, Phys<R> p, const R* Tin, R* Tout)
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
-    chain_next();
     chain_wait();
     if (x >= g.nx || y >= g.ny) return;
     const int nx = g.nx, ny = g.ny, nz = g.nz, pitch = g.pitch;
