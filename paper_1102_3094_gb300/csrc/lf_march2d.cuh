@@ -381,6 +381,22 @@ inline int march2_rows_for(int nx, int ny, int U, int param, int sms)
     return best;
 }
 
+// CTAs per SM to leave room for: what an even spread of a march's grid gives
+// when that is below the `most` that fit, else 0 (no preference).  A grid that
+// is let in while its predecessor drains would otherwise fill the SMs that are
+// free first: FP32 2999 x 1777 after its temperature sub-steps 147 us a step,
+// 114 with two CTAs per SM.  FP64 CTAs of 128 threads, four for every SM, run
+// as two rounds of two instead of three and then one: 1500 x 1200 720 us against
+// 967, 2048 x 1024 844 / 982, without hydrodynamics 143 / 190.  With more of them
+// or with 64 threads the full SM is the better one: 2048^2 without hydrodynamics
+// 287 us against 308 at two CTAs, 512^2 on 64 threads and 16 rows 172 / 235.
+inline int spread(int element_bytes, int threads, int most, unsigned grid_x, unsigned grid_y, int sms)
+{
+    const int64_t k = ((int64_t)grid_x * grid_y + sms - 1) / sms;
+    if (k < most) return (int)k;
+    return element_bytes == 8 && threads == 128 && k == 4 ? 2 : 0;
+}
+
 // CTA width and rows per lane of the two-lane (packed FP32) marches.  A CTA of
 // 64 threads (56 columns) or 128 (120) brings two or four warps, and an SM's
 // four schedulers take three warps each (six or three CTAs, by registers).

@@ -98,20 +98,6 @@ __global__ void __launch_bounds__(NT, MINB) k_march2d_x2(Geom g, Phys<float> p, 
     chain_next();
 }
 
-// CTAs per SM to leave room for: what an even spread of a march's grid gives
-// when that is below the `most` that fit, else 0 (no preference).  A grid that
-// is let in while its predecessor drains would otherwise fill the SMs that are
-// free first: 2999 x 1777 after its temperature sub-steps 147 us a step, 114
-// with two CTAs per SM.  FP64 marches, bound by their pipe, take at most two
-// (512^2: 242 -> 174 us, 1024^2 the same).
-template <typename R>
-int spread_of(dim3 grid, int sms, int most = sizeof(R) == 4 ? 3 : 2)
-{
-    const int64_t k = ((int64_t)grid.x * grid.y + sms - 1) / sms;
-    if (sizeof(R) == 8) return k < most ? (int)k : most;
-    return k < most ? (int)k : 0;
-}
-
 template <int NT, int D, bool HYDRO, int MINB>
 cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<float>& io, int H, int sms, cudaStream_t s)
 {
@@ -123,7 +109,7 @@ cudaError_t launch_march_x2(const Geom& g, const Phys<float>& p, const StepIO<fl
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms, NT == 64 ? 6 : 3), s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, march::spread(4, NT, NT == 64 ? 6 : 3, grid.x, grid.y, sms), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -138,7 +124,7 @@ cudaError_t launch_march(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<R>(grid, sms), s, g, p, io, H);
+    return launch_chained(kern, grid, NT, M::BYTES, march::spread(sizeof(R), NT, sizeof(R) == 8 && NT == 64 ? 4 : 3, grid.x, grid.y, sms), s, g, p, io, H);
 }
 
 template <int NT, int D, bool HYDRO, int MINB>
@@ -152,7 +138,7 @@ cudaError_t launch_march_iso_x2(const Geom& g, const Phys<float>& p, const StepI
     int npairs = (g.ny + 2 * H - 1) / (2 * H);
     if (npairs > g.ny / 2) npairs = g.ny / 2;       // every lane keeps at least one row
     dim3 grid((g.nx + M::U - 1) / M::U, npairs);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<float>(grid, sms, NT == 64 ? 6 : 3), s, g, p, io, npairs);
+    return launch_chained(kern, grid, NT, M::BYTES, march::spread(4, NT, NT == 64 ? 6 : 3, grid.x, grid.y, sms), s, g, p, io, npairs);
 }
 
 template <typename R, int NT, int D>
@@ -167,7 +153,7 @@ cudaError_t launch_march_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int H = march::march2_rows_for(g.nx, g.ny, M::U, g.tune & 0xFFFF, sms);
     dim3 grid((g.nx + M::U - 1) / M::U, (g.ny + H - 1) / H);
-    return launch_chained(kern, grid, NT, M::BYTES, spread_of<R>(grid, sms), s, g, p, io, H);
+    return launch_chained(kern, grid, NT, M::BYTES, march::spread(sizeof(R), NT, sizeof(R) == 8 && NT == 64 ? 4 : 3, grid.x, grid.y, sms), s, g, p, io, H);
 }
 
 // The two-lane marches: width and rows per lane by march::pair_shape.

@@ -1,0 +1,54 @@
+"""The rules that choose launch shapes (csrc/lf_march2d.cuh), compiled for the
+host."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.join(os.path.dirname(__file__), "..")
+NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+
+PROGRAM = r"""
+#include "lf_march2d.cuh"
+#include <cstdio>
+#include <cstring>
+using namespace lf;
+int main()
+{
+    char what[16];
+    int a[6];
+    while (std::scanf("%15s %d %d %d %d %d %d", what, a, a + 1, a + 2, a + 3, a + 4, a + 5) == 7) {
+        if (!std::strcmp(what, "spread")) std::printf("%d\n", march::spread(a[0], a[1], a[2], a[3], a[4], a[5]));
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def ask(tmp_path_factory):
+    if not os.path.exists(NVCC):
+        pytest.skip("needs nvcc")
+    d = tmp_path_factory.mktemp("shape")
+    (d / "p.cu").write_text(PROGRAM)
+    subprocess.run([NVCC, "-std=c++17", "-O2", "-gencode", "arch=compute_103a,code=sm_103a", "--expt-relaxed-constexpr",
+                    "-I", os.path.join(ROOT, "include"), "-I", os.path.join(ROOT, "paper_1102_3094_gb300", "csrc"),
+                    str(d / "p.cu"), "-o", str(d / "p")], check=True)
+
+    def run(*queries):
+        text = "".join(" ".join(map(str, list(q) + [0] * (7 - len(q)))) + "\n" for q in queries)
+        out = subprocess.run([str(d / "p")], input=text, capture_output=True, text=True, check=True).stdout
+        return [[float(v) for v in line.split()] for line in out.splitlines()]
+
+    return run
+
+
+@pytest.mark.parametrize("element_bytes,threads,most,per_sm,want", [
+    (4, 128, 3, 1, 1), (4, 128, 3, 2, 2), (4, 128, 3, 3, 0), (4, 128, 3, 4, 0), (4, 64, 6, 5, 5), (4, 64, 6, 6, 0),
+    # FP64: two rounds of two; more rounds, or 64 threads, take what fits
+    (8, 128, 3, 1, 1), (8, 128, 3, 2, 2), (8, 128, 3, 3, 0), (8, 128, 3, 4, 2), (8, 128, 3, 5, 0), (8, 128, 3, 6, 0),
+    (8, 64, 4, 2, 2), (8, 64, 4, 3, 3), (8, 64, 4, 4, 0), (8, 64, 4, 8, 0)])
+def test_spread_of_a_march(ask, element_bytes, threads, most, per_sm, want):
+    # the last SM's share may be short
+    for ctas in (152 * per_sm, 152 * (per_sm - 1) + 1):
+        assert ask(("spread", element_bytes, threads, most, ctas, 1, 152)) == [[want]]
