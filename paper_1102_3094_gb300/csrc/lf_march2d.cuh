@@ -3,6 +3,8 @@
 // ensemble kernel (lf_ens.cu), so both run exactly the same arithmetic.
 #pragma once
 
+#include <algorithm>
+
 #include "lf_internal.cuh"
 
 namespace lf {
@@ -417,6 +419,11 @@ struct PairShape {
     int rows;
 };
 
+constexpr int kPairPasses = 6;                      // full passes a shape may take: more never won over 20,000 sizes
+
+// The search goes over k, not over heights: at one k the shortest lanes win, so
+// each k has one candidate.  (A search over up to 512 heights took the host 0.8
+// us of every step at 1024^2 and 7 at 4096^2, this one 0.4, with the same result.)
 inline PairShape pair_shape(int nx, int ny, int tune, bool iso, int sms)
 {
     const int fixed = tune & 0xFFFF, width = tune >> 16;
@@ -427,21 +434,24 @@ inline PairShape pair_shape(int nx, int ny, int tune, bool iso, int sms)
     float best_us = -1.f;
     for (int narrow = width == 1 ? 1 : 0; narrow < 2; ++narrow) {
         const int U = narrow ? 56 : 120, strips = (nx + U - 1) / U;
-        for (int h = 1; h <= ny && h <= 512; ++h) {
-            int pairs = (ny + 2 * h - 1) / (2 * h);
-            if (pairs > ny / 2) pairs = ny / 2;     // every lane keeps at least one row
-            if (pairs < 1) break;
-            const int l = (ny + 2 * pairs - 1) / (2 * pairs);
-            const int64_t per_sm = ((int64_t)strips * pairs + sms - 1) / sms;
-            const int64_t k = narrow ? (per_sm + 1) / 2 : per_sm;
+        const int64_t places = (int64_t)sms * (narrow ? 2 : 1);         // CTAs per k
+        for (int64_t kmax = 1; kmax <= 3 * kPairPasses; ++kmax) {
+            int64_t pairs = kmax * places / strips;
+            if (pairs > ny / 2) pairs = ny / 2;         // every lane keeps at least one row
+            if (pairs < 1) continue;
+            const int64_t least = (ny + 2 * pairs - 1) / (2 * pairs);
+            const int l = least < 512 ? (int)least : 512;               // no measurements of taller ones
+            const int rows = pairs == ny / 2 ? 1 : l;
+            const int64_t ctas = strips * std::min<int64_t>(((int64_t)ny + 2 * rows - 1) / (2 * rows), ny / 2);
+            const int64_t k = (ctas + places - 1) / places;
             float us = 3.f + (float)(k / 3) * (row[iso][3] * l + lag[iso][3]);
             if (k % 3) us += row[iso][k % 3] * l + lag[iso][k % 3];
             if (narrow) us *= 0.98f;
             if (best_us < 0.f || us < best_us) {
                 best_us = us;
-                best = {narrow == 1, h};
+                best = {narrow == 1, rows};
             }
-            if (per_sm == 1) break;                 // taller lanes only take longer
+            if (pairs == ny / 2) break;                 // more CTAs are not to be had
         }
     }
     return best;

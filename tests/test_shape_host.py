@@ -11,14 +11,30 @@ NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
 
 PROGRAM = r"""
 #include "lf_march2d.cuh"
+#include <algorithm>
+#include <chrono>
 #include <cstdio>
 #include <cstring>
 using namespace lf;
+
+static double us_per_call(int nx, int ny, bool iso)
+{
+    double best = 1e9;
+    for (int batch = 0; batch < 20; ++batch) {
+        const auto t = std::chrono::steady_clock::now();
+        volatile int sink = 0;
+        for (int i = 0; i < 500; ++i) sink = sink + march::pair_shape(nx, ny, 0, iso, 152).rows;
+        best = std::min(best, std::chrono::duration<double>(std::chrono::steady_clock::now() - t).count() / 500 * 1e6);
+    }
+    return best;
+}
+
 int main()
 {
     char what[16];
     int a[6];
     while (std::scanf("%15s %d %d %d %d %d %d", what, a, a + 1, a + 2, a + 3, a + 4, a + 5) == 7) {
+        if (!std::strcmp(what, "time")) std::printf("%f\n", us_per_call(a[0], a[1], a[2] != 0));
         if (!std::strcmp(what, "spread")) std::printf("%d\n", march::spread(a[0], a[1], a[2], a[3], a[4], a[5]));
     }
 }
@@ -52,3 +68,10 @@ def test_spread_of_a_march(ask, element_bytes, threads, most, per_sm, want):
     # the last SM's share may be short
     for ctas in (152 * per_sm, 152 * (per_sm - 1) + 1):
         assert ask(("spread", element_bytes, threads, most, ctas, 1, 152)) == [[want]]
+
+
+@pytest.mark.parametrize("nx,ny", [(256, 256), (1024, 1024), (2999, 1777), (4096, 4096), (32, 100000)])
+def test_a_shape_is_cheap_to_choose(ask, nx, ny):
+    """lf_step chooses it for every step: well under the launch itself (a few microseconds)."""
+    for iso in (0, 1):
+        assert ask(("time", nx, ny, iso))[0][0] < 2.0
