@@ -412,8 +412,13 @@ inline int spread(int element_bytes, int threads, int most, unsigned grid_x, uns
 // within 0.2 % of the best measured shape on average (2 % at worst); against
 // (CTAs per SM) x (l + 4) on 128 threads: 256^2 8.5 -> 7.4 us a step, 512^2
 // 13.4 -> 12.0, 1024^2 25.4 -> 24.4, isotropic 384^2 15.7 -> 13.1, 1024^2
-// 35.9 -> 32.8, 2999 x 1777 133.6 -> 120.  The tuner's param names a height
-// (low 16 bits) and 64 threads (bit 16); a height alone means 128 threads.
+// 35.9 -> 32.8, 2999 x 1777 133.6 -> 120.  Without hydrodynamics the compact
+// rows are a third of that and three warps per scheduler pay (0.42 / 0.56 / 0.60
+// us a row and 2 us, over 24 sizes from 64^2 to 8192 x 4096: 0.6 % from the best
+// shape, 5 % at worst): with the constants above 1024^2 took 11.9 us, now 10.2,
+// 2048^2 39.4 / 30.6; the isotropic choice is the best one with the same constants
+// (0.7 %).  The tuner's param names a height (low 16 bits) and 64 threads (bit 16);
+// a height alone means 128 threads.
 struct PairShape {
     bool narrow;                                    // 64 threads
     int rows;
@@ -424,12 +429,14 @@ constexpr int kPairPasses = 6;                      // full passes a shape may t
 // The search goes over k, not over heights: at one k the shortest lanes win, so
 // each k has one candidate.  (A search over up to 512 heights took the host 0.8
 // us of every step at 1024^2 and 7 at 4096^2, this one 0.4, with the same result.)
-inline PairShape pair_shape(int nx, int ny, int tune, bool iso, int sms)
+inline PairShape pair_shape(int nx, int ny, int tune, bool iso, bool hydro, int sms)
 {
     const int fixed = tune & 0xFFFF, width = tune >> 16;
     if (fixed > 0) return {width == 1, fixed < ny ? fixed : ny};
-    const float row[2][4] = {{0, 1.10f, 1.24f, 1.89f}, {0, 1.33f, 1.70f, 2.15f}};
-    const float lag[2][4] = {{0, 2.6f, 3.0f, 3.4f}, {0, 5.0f, 5.5f, 6.4f}};
+    const float rows_us[3][4] = {{0, 1.10f, 1.24f, 1.89f}, {0, 1.33f, 1.70f, 2.15f}, {0, 0.42f, 0.56f, 0.60f}};
+    const float lag_us[3][4] = {{0, 2.6f, 3.0f, 3.4f}, {0, 5.0f, 5.5f, 6.4f}, {0, 0.6f, 0.6f, 1.2f}};
+    const int form = iso ? 1 : hydro ? 0 : 2;
+    const float *row = rows_us[form], *lag = lag_us[form], launch = form == 2 ? 2.f : 3.f;
     PairShape best{width == 1, 1};
     float best_us = -1.f;
     for (int narrow = width == 1 ? 1 : 0; narrow < 2; ++narrow) {
@@ -444,8 +451,8 @@ inline PairShape pair_shape(int nx, int ny, int tune, bool iso, int sms)
             const int rows = pairs == ny / 2 ? 1 : l;
             const int64_t ctas = strips * std::min<int64_t>(((int64_t)ny + 2 * rows - 1) / (2 * rows), ny / 2);
             const int64_t k = (ctas + places - 1) / places;
-            float us = 3.f + (float)(k / 3) * (row[iso][3] * l + lag[iso][3]);
-            if (k % 3) us += row[iso][k % 3] * l + lag[iso][k % 3];
+            float us = launch + (float)(k / 3) * (row[3] * l + lag[3]);
+            if (k % 3) us += row[k % 3] * l + lag[k % 3];
             if (narrow) us *= 0.98f;
             if (best_us < 0.f || us < best_us) {
                 best_us = us;

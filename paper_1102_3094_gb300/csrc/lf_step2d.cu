@@ -164,7 +164,7 @@ cudaError_t launch_pair_shape(const Geom& g, const Phys<float>& p, const StepIO<
     const cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
     const bool iso = g.stencil == LF_STENCIL_ISOTROPIC;
-    const march::PairShape c = march::pair_shape(g.nx, g.ny, g.tune, iso, sms);
+    const march::PairShape c = march::pair_shape(g.nx, g.ny, g.tune, iso, HYDRO, sms);
     if (iso)
         return c.narrow ? launch_march_iso_x2<64, 3, HYDRO, 6>(g, p, io, c.rows, sms, s)
                         : launch_march_iso_x2<128, 3, HYDRO, 3>(g, p, io, c.rows, sms, s);

@@ -23,7 +23,7 @@ static double us_per_call(int nx, int ny, bool iso)
     for (int batch = 0; batch < 20; ++batch) {
         const auto t = std::chrono::steady_clock::now();
         volatile int sink = 0;
-        for (int i = 0; i < 500; ++i) sink = sink + march::pair_shape(nx, ny, 0, iso, 152).rows;
+        for (int i = 0; i < 500; ++i) sink = sink + march::pair_shape(nx, ny, 0, iso, true, 152).rows;
         best = std::min(best, std::chrono::duration<double>(std::chrono::steady_clock::now() - t).count() / 500 * 1e6);
     }
     return best;
@@ -35,6 +35,10 @@ int main()
     int a[6];
     while (std::scanf("%15s %d %d %d %d %d %d", what, a, a + 1, a + 2, a + 3, a + 4, a + 5) == 7) {
         if (!std::strcmp(what, "time")) std::printf("%f\n", us_per_call(a[0], a[1], a[2] != 0));
+        if (!std::strcmp(what, "pair")) {
+            const march::PairShape c = march::pair_shape(a[0], a[1], a[2], a[3] != 0, a[4] != 0, 152);
+            std::printf("%d %d\n", c.narrow, c.rows);
+        }
         if (!std::strcmp(what, "spread")) std::printf("%d\n", march::spread(a[0], a[1], a[2], a[3], a[4], a[5]));
     }
 }
@@ -75,3 +79,13 @@ def test_a_shape_is_cheap_to_choose(ask, nx, ny):
     """lf_step chooses it for every step: well under the launch itself (a few microseconds)."""
     for iso in (0, 1):
         assert ask(("time", nx, ny, iso))[0][0] < 2.0
+
+
+@pytest.mark.parametrize("nx,ny", [(700, 611), (1024, 1024), (2048, 512), (512, 2048), (1400, 1300), (1800, 1900), (2048, 2048),
+                                   (3000, 1500), (2500, 2400), (3000, 3000), (300, 5000)])
+def test_compact_march_without_hydrodynamics_fills_the_schedulers(ask, nx, ny):
+    """Measured best at every one of these: lanes so short that three warps per scheduler hold the lattice."""
+    (narrow, rows), = ask(("pair", nx, ny, 0, 0, 0))
+    strips, places = -(-nx // (56 if narrow else 120)), 152 * (2 if narrow else 1)
+    ctas = strips * -(-ny // int(2 * rows))
+    assert 2 * places < ctas <= 3 * places
