@@ -224,8 +224,10 @@ __device__ __forceinline__ double kfreq2(int i, int n, int64_t lmin)
 // from a table, and the shell b = floor(sqrt(r2) + 1/2) from an FP32 root
 // corrected against (b - 1/2)^2 <= r2 < (b + 1/2)^2 in FP64: about ten FP64
 // operations per mode (the divisions and the FP64 root made it sixty): 114 ->
-// 32 us at 1024^2.
-__global__ void __launch_bounds__(kThreads) k_shells(Geom g, const double2* __restrict__ X, int64_t lmin, int B,
+// 32 us at 1024^2.  A lattice of few rows is cut into `parts` parts of a row, a
+// multiple of 32 modes each: 4096 x 64 had eight CTAs, whose lanes add to the same
+// shell one after the other (298 us; 40 with parts on every SM).
+__global__ void __launch_bounds__(kThreads) k_shells(Geom g, const double2* __restrict__ X, int64_t lmin, int B, int parts,
                                                      double* __restrict__ bins)
 {
     extern __shared__ double sm[];
@@ -237,15 +239,17 @@ __global__ void __launch_bounds__(kThreads) k_shells(Geom g, const double2* __re
     for (int i = threadIdx.x; i < H; i += kThreads) kx2[i] = kfreq2(i, g.nx, lmin);
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int rows = g.ny * g.nz, step = gridDim.x * (kThreads / 32);
+    const int items = g.ny * g.nz * parts, step = gridDim.x * (kThreads / 32);
+    const int span = ((H + 31) / 32 + parts - 1) / parts * 32;
     const double top = ((double)B + 0.5) * ((double)B + 0.5);
-    for (int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows; row += step) {
+    for (int it = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); it < items; it += step) {
+        const int row = it / parts, beg = (it - row * parts) * span, end = min(beg + span, H);
         const int iz = row / g.ny, iy = row - iz * g.ny;
         double rr = kfreq2(iy, g.ny, lmin);
         if (g.d == 3) rr += kfreq2(iz, g.nz, lmin);
         if (rr >= top) continue;
         const double2* x = X + (int64_t)row * H;
-        for (int ix = lane; ix < H; ix += 32) {
+        for (int ix = beg + lane; ix < end; ix += 32) {
             const double r2 = kx2[ix] + rr;
             if (r2 >= top) break;
             int b = (int)(sqrtf((float)r2) + 0.5f);
@@ -304,9 +308,11 @@ bool enqueue_sk(const DiagInput& in, const Scratch& sc, cudaStream_t s, cudaErro
     static unsigned long long attr_done = 0;
     const int most = (int)((sizeof(double) + sizeof(unsigned)) * (kMaxBins + 1) + sizeof(double) * (kMaxBins + 1));
     if ((*err = raise_smem_limit(k_shells, most, &attr_done)) != cudaSuccess) return true;
-    const int64_t warps = (int64_t)g.ny * g.nz;
-    const unsigned nblk = (unsigned)std::min<int64_t>(152 * 4, (warps + kThreads / 32 - 1) / (kThreads / 32));
-    k_shells<<<nblk, kThreads, hs, s>>>(g, sc.fft, lmin, (int)B, sc.bins);
+    // about one CTA for every SM where whole rows give fewer, as far as parts of 32 modes go
+    const int64_t rows = (int64_t)g.ny * g.nz, cta = kThreads / 32;
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(152 * cta / rows, (half_nx(g.nx) + 31) / 32));
+    const unsigned nblk = (unsigned)std::min<int64_t>(152 * 4, (rows * parts + cta - 1) / cta);
+    k_shells<<<nblk, kThreads, hs, s>>>(g, sc.fft, lmin, (int)B, parts, sc.bins);
     *err = cudaGetLastError();
     return true;
 }
