@@ -1,4 +1,5 @@
 // lf_util.cu -- initial state and layout conversion kernels.
+#include "lf_cvt.h"
 #include "lf_internal.cuh"
 
 namespace lf {
@@ -57,7 +58,7 @@ __global__ void k_init(Geom g, uint64_t seed, double amp, double T0, double T_w,
 // The offset w_i n0 is added in the arithmetic of the caller's type.  The
 // FP64 pipe of this GPU issues 1.8 operations per clock and SM (FP32: 118), and
 // converting FP32 state through it made this kernel three FP64 operations per
-// element, 0.41 G elements/ms whatever the bandwidth.  FP32 to FP32 therefore
+// element, 0.16 G elements/ms whatever the bandwidth.  FP32 to FP32 therefore
 // adds the offset as three floats (24 + 24 + 5 bits hold the double exactly)
 // with error-free sums: the result is the sum rounded once, to within 2^-46
 // relative, as (float)((double)v + a) is.  19 populations at 384^3: 6.6 ms
@@ -151,12 +152,12 @@ __global__ void __launch_bounds__(256) k_convert(const S* __restrict__ src, D* _
     const int q = blockIdx.y;
     src += q * sp;
     dst += q * dp;
-    const unsigned g0 = blockIdx.x * (256u * kGroups) + threadIdx.x;
+    const unsigned nt = blockDim.x, g0 = blockIdx.x * (nt * kGroups) + threadIdx.x;
     S v[kGroups][V];
     int64_t to[kGroups];
 #pragma unroll
     for (int u = 0; u < kGroups; ++u) {
-        const unsigned k = g0 + 256u * u;
+        const unsigned k = g0 + nt * u;
         if (k < groups) {
             const unsigned row = k / row_groups, x = (k - row * row_groups) * V;
             to[u] = row * drow + x;
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(256) k_convert(const S* __restrict__ src, D* _
     }
 #pragma unroll
     for (int u = 0; u < kGroups; ++u)
-        if (g0 + 256u * u < groups) {
+        if (g0 + nt * u < groups) {
             D o[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) o[i] = add_offset<S, D>(v[u][i], off, q);
@@ -189,11 +190,19 @@ cudaError_t convert(const Geom& g, const S* src, D* dst, int nplanes, int64_t sr
                     bool vec, const Offsets& off, cudaStream_t s)
 {
     // sites < 2^31 / Q (checked at creation), so groups fit 32 bits
+    int sms = 0;
+    const cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    // Small planes: one element per group and small blocks, because a thread that converts four between FP32 and FP64
+    // is a chain on the FP64 pipe of one SM.  64 x 64 populations and a host array of the other type, one plane at a
+    // time: read 138 -> 128 us, written 68.5 -> 64.5.
+    if ((uint64_t)g.nx * g.ny * g.nz * nplanes < 256ull * sms) vec = false;
     const unsigned row_groups = vec ? g.nx / 4 : g.nx;
     const unsigned groups = row_groups * (unsigned)(g.ny * g.nz);
-    const dim3 grid((groups + 256 * kGroups - 1) / (256 * kGroups), nplanes);
-    if (vec) k_convert<S, D, 4><<<grid, 256, 0, s>>>(src, dst, groups, row_groups, srow, drow, sp, dp, off);
-    else k_convert<S, D, 1><<<grid, 256, 0, s>>>(src, dst, groups, row_groups, srow, drow, sp, dp, off);
+    const unsigned nt = convert_threads(groups, kGroups, nplanes, sms), per = nt * kGroups;
+    const dim3 grid((groups + per - 1) / per, nplanes);
+    if (vec) k_convert<S, D, 4><<<grid, nt, 0, s>>>(src, dst, groups, row_groups, srow, drow, sp, dp, off);
+    else k_convert<S, D, 1><<<grid, nt, 0, s>>>(src, dst, groups, row_groups, srow, drow, sp, dp, off);
     return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
-"""The rules that choose launch shapes (csrc/lf_march2d.cuh), compiled for the
-host."""
+"""The rules that choose launch shapes (csrc/lf_march2d.cuh, csrc/lf_cvt.h),
+compiled for the host."""
 import os
 import shutil
 import subprocess
@@ -11,6 +11,7 @@ NVCC = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
 
 PROGRAM = r"""
 #include "lf_march2d.cuh"
+#include "lf_cvt.h"
 #include <algorithm>
 #include <chrono>
 #include <cstdio>
@@ -35,6 +36,7 @@ int main()
     int a[6];
     while (std::scanf("%15s %d %d %d %d %d %d", what, a, a + 1, a + 2, a + 3, a + 4, a + 5) == 7) {
         if (!std::strcmp(what, "time")) std::printf("%f\n", us_per_call(a[0], a[1], a[2] != 0));
+        if (!std::strcmp(what, "convert")) std::printf("%u\n", convert_threads(a[0], a[1], a[2], a[3]));
         if (!std::strcmp(what, "pair")) {
             const march::PairShape c = march::pair_shape(a[0], a[1], a[2], a[3] != 0, a[4] != 0, 152);
             std::printf("%d %d\n", c.narrow, c.rows);
@@ -89,3 +91,10 @@ def test_compact_march_without_hydrodynamics_fills_the_schedulers(ask, nx, ny):
     strips, places = -(-nx // (56 if narrow else 120)), 152 * (2 if narrow else 1)
     ctas = strips * -(-ny // int(2 * rows))
     assert 2 * places < ctas <= 3 * places
+
+
+@pytest.mark.parametrize("groups,planes,want", [(1, 1, 32), (1024, 1, 32), (1024, 9, 32), (8192, 9, 32), (16384, 9, 64),
+                                                (34304, 9, 128), (69376, 9, 256), (311296, 1, 256), (310784, 1, 128), (1 << 29, 1, 256)])
+def test_a_small_conversion_is_spread_over_the_sms(ask, groups, planes, want):
+    """Two groups per thread and 152 SMs: the largest block that gives every SM four, 32 threads at least."""
+    assert ask(("convert", groups, 2, planes, 152)) == [[want]]
