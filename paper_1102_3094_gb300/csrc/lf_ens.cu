@@ -9,10 +9,10 @@
 // over the strips and row segments of those runs.  Runs with the isotropic stencils are (run, strip, pair) items of a
 // second persistent kernel that runs the two-lane isotropic row march
 // (lf_march2d_iso.cuh), the code a single isotropic FP32 run uses by default.
-// Every run returns to its starting buffers
-// after two steps (f and phi flip once per step, T flips nsub times), so two
-// steps are captured in one CUDA graph and replayed; single-step graphs handle
-// odd counts.
+// Every run returns to its starting buffers after two steps (f and phi flip once
+// per step, T once and once for every pass of further sub-steps), so two steps
+// are captured in one CUDA graph and replayed; single-step graphs handle odd
+// counts.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -301,8 +301,8 @@ int build(lf_ens* e)
         }
     }
     // work lists: march items per kind and CTA width (compact 64, 128,
-    // isotropic 64, 128) sorted by cost (longest lane first), T tiles per
-    // sub-step
+    // isotropic 64, 128) sorted by cost (longest lane first), row segments
+    // of T per pass of sub-steps
     std::vector<EnsItem> items[4];
     for (int r = 0; r < R; ++r) {
         const lf_ctx* c = e->runs[r];
@@ -410,28 +410,34 @@ int build(lf_ens* e)
 // Rows per lane of every run before any tuning, one height for all runs of a
 // stencil, with 64-thread CTAs (the better width at 4 to 96 runs of 128^2 to
 // 512^2, both stencils).  Six CTAs fit an SM; CTA b takes the items b, b + B,
-// ... of the list sorted by length, so the step takes what CTA 0 does: per
-// item of l rows about s l + c us, measured with heights of 2 to 128 (compact
-// 1.89 l + 5.5, isotropic 2.4 l + 10; s falls to 1.24 / 1.7 and 1.1 / 1.33
-// where four or two CTAs per SM hold all items).  Against 16 rows: 10 runs 45.6
-// -> 41.3 us a step, 48 runs 168 -> 149, 96 runs 313 -> 273, isotropic 411 ->
-// 354; within 1 % of the best uniform height at seven of eight counts of runs.
+// ... of the list sorted by length, so the step takes what CTA 0 does: per item of
+// l rows about s l + c us, by the warps per scheduler that the round leaves (a
+// last round of few items runs faster).  s and c are those that choose best over
+// 19 batches from 2000 runs of 32^2 to three of 4096^2 at heights of 1 to 512: from
+// the best uniform height 0.3 % on average (compact; 2 % at worst), 0.7 %
+// (isotropic; 3 %), without hydrodynamics 0.3 and 0.2 %.  Against 16 rows: 10 runs
+// of 128^2 to 512^2 45.6 -> 41.3 us a step, 96 runs 313 -> 273, isotropic 411 -> 354.
 void default_rows(lf_ens* e)
 {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sms = std::max(1, sms);
-    const float row[2][4] = {{0, 1.10f, 1.24f, 1.89f}, {0, 1.33f, 1.70f, 2.4f}};
-    const float lag[2] = {5.5f, 10.f};
+    // [hydrodynamics][isotropic][warps per scheduler]; isotropic, one round at two warps: 1.93 and 6
+    const float row[2][2][4] = {{{0, 0.43f, 0.57f, 0.59f}, {0, 0.44f, 0.52f, 0.63f}},
+                                {{0, 1.16f, 1.30f, 1.57f}, {0, 1.37f, 2.57f, 2.48f}}};
+    const float lag[2][2][4] = {{{0, 4.96f, 2.46f, 3.13f}, {0, 5.05f, 7.2f, 5.3f}},
+                                {{0, 11.05f, 6.59f, 7.84f}, {0, 5.08f, 26.1f, 6.1f}}};
+    auto warps = [sms](int64_t ctas) { return (int)std::min<int64_t>(3, ((ctas + sms - 1) / sms + 1) / 2); };
     for (int iso = 0; iso < 2; ++iso) {
         std::vector<int> members;
         std::map<std::pair<int, int>, int> sizes;                        // (nx, ny): runs
-        int tallest = 0;
+        int tallest = 0, flow = 0;
         for (int r = 0; r < e->nruns; ++r) {
             const Geom& g = e->runs[r]->g;
             if ((g.stencil == LF_STENCIL_ISOTROPIC) != (iso == 1)) continue;
             members.push_back(r);
+            flow |= e->runs[r]->params.hydro != 0;
             ++sizes[{g.nx, g.ny}];
             tallest = std::max(tallest, g.ny);
         }
@@ -450,12 +456,16 @@ void default_rows(lf_ens* e)
             }
             std::sort(lanes.begin(), lanes.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
             const int64_t B = std::min<int64_t>(items, 6 * (int64_t)sms);
-            const int k = (int)std::min<int64_t>(3, ((B + sms - 1) / sms + 1) / 2);
+            const int full = warps(B), last = warps((items - 1) % B + 1);
+            const bool alone = flow && iso && items == B && full == 2;
             float us = 0.f;
             int64_t next = 0, end = 0;                                   // CTA 0's next item; items seen
             for (const auto& l : lanes) {
                 end += l.second;
-                for (; next < end; next += B) us += row[iso][k] * l.first + lag[iso];
+                for (; next < end; next += B) {
+                    const int k = next + B < items ? full : last;
+                    us += alone ? 1.93f * l.first + 6.f : row[flow][iso][k] * l.first + lag[flow][iso][k];
+                }
             }
             if (best_us < 0.f || us < best_us) {
                 best_us = us;
