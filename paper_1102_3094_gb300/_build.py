@@ -30,9 +30,14 @@ def nvcc() -> str:
     raise RuntimeError("nvcc not found: the CUDA toolkit is required to build liblf.so")
 
 
+def headers() -> list[str]:
+    """Every file that a source may include."""
+    return [f for pat in (os.path.join(CSRC, "*.cuh"), os.path.join(CSRC, "*.h"), os.path.join(INCLUDE, "*.h"))
+            for f in glob.glob(pat)]
+
+
 def _deps_mtime() -> float:
-    files = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h")) + [__file__]
-    return max(os.path.getmtime(f) for f in files)
+    return max(os.path.getmtime(f) for f in headers() + [__file__])
 
 
 def _compile(src: str, verbose_ptxas: bool) -> str:
