@@ -220,26 +220,28 @@ int capture(lf_ens* e, const std::vector<int>& halves, const Half* H, const std:
 {
     cudaGraph_t graph;
     if (cudaStreamBeginCapture(e->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return LF_ECUDA;
+    cudaError_t launched = cudaSuccess;          // one refused for its attributes does not invalidate the capture
+    auto add = [&](auto kern, int blocks, int threads, size_t smem, int spread, auto... args) {
+        if (launched == cudaSuccess) launched = launch_chained(kern, blocks, threads, smem, spread, e->stream, args...);
+    };
     for (int h : halves) {
-        if (e->nitems[0] > 0)
-            launch_chained(kEns64, e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->spread[0], e->stream, H[h].runs,
-                           e->d_items[0], e->nitems[0]);
-        if (e->nitems[1] > 0)
-            launch_chained(kEns128, e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->spread[1], e->stream, H[h].runs,
-                           e->d_items[1], e->nitems[1]);
-        if (e->nitems[2] > 0)
-            launch_chained(kIso64, e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->spread[2], e->stream, H[h].runs,
-                           e->d_items[2], e->nitems[2]);
-        if (e->nitems[3] > 0)
-            launch_chained(kIso128, e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->spread[3], e->stream, H[h].runs,
-                           e->d_items[3], e->nitems[3]);
-        for (size_t s = 0; s < H[h].ts.size(); ++s) {
-            if (ntitems[s] == 0) continue;
-            launch_chained(k_ens_tsub2d, (ntitems[s] + 3) / 4, 128, 0, e->stream, H[h].ts[s], titems[s], ntitems[s]);
-        }
+        const EnsRun* runs = H[h].runs;
+        if (e->nitems[0] > 0) add(kEns64, e->march_blocks[0], 64, MarchCfg<64>::BYTES, e->spread[0], runs, e->d_items[0], e->nitems[0]);
+        if (e->nitems[1] > 0) add(kEns128, e->march_blocks[1], 128, MarchCfg<128>::BYTES, e->spread[1], runs, e->d_items[1], e->nitems[1]);
+        if (e->nitems[2] > 0) add(kIso64, e->march_blocks[2], 64, IsoCfg<64>::BYTES, e->spread[2], runs, e->d_items[2], e->nitems[2]);
+        if (e->nitems[3] > 0) add(kIso128, e->march_blocks[3], 128, IsoCfg<128>::BYTES, e->spread[3], runs, e->d_items[3], e->nitems[3]);
+        for (size_t s = 0; s < H[h].ts.size(); ++s)
+            if (ntitems[s] > 0) add(k_ens_tsub2d, (ntitems[s] + 3) / 4, 128, 0, 0, H[h].ts[s], titems[s], ntitems[s]);
     }
-    cudaError_t err = cudaStreamEndCapture(e->stream, &graph);   // reports a failed launch too
-    if (err != cudaSuccess) return LF_ECUDA;
+    cudaError_t err = cudaStreamEndCapture(e->stream, &graph);
+    if (err == cudaSuccess && launched != cudaSuccess) {
+        cudaGraphDestroy(graph);
+        err = launched;
+    }
+    if (err != cudaSuccess) {
+        cudaGetLastError();
+        return LF_ECUDA;
+    }
     err = cudaGraphInstantiate(out, graph, 0);
     cudaGraphDestroy(graph);
     return err == cudaSuccess ? LF_OK : LF_ECUDA;

@@ -252,7 +252,7 @@ __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.laun
 // `spread` > 0: the share of the L1 that becomes shared memory is what `spread`
 // CTAs of this kernel need, not what most would.
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, int spread, cudaStream_t s, const A&... args)
+[[nodiscard]] cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, int spread, cudaStream_t s, const A&... args)
 {
     cudaLaunchAttribute at[2] = {};
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -271,7 +271,7 @@ cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t sme
 }
 
 template <typename... P, typename... A>
-cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args)
+[[nodiscard]] cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args)
 {
     return launch_chained(kern, grid, block, smem, 0, s, args...);
 }

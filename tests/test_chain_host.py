@@ -73,3 +73,11 @@ def test_no_restrict_outside_kernel_parameters(path):
     for _, params, _ in kernels(text):
         text = text.replace(params, "")
     assert "__restrict__" not in text
+
+
+@pytest.mark.parametrize("path", files(), ids=os.path.basename)
+def test_no_launch_status_is_dropped(path):
+    """A launch that is refused (its configuration or attributes) only says so in what launch_chained returns; under
+    capture a graph would go without that kernel."""
+    text = source(path)
+    assert not re.search(r"[;{})]\s*launch_chained\(", text)
