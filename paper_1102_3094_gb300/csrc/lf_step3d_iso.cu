@@ -778,7 +778,8 @@ cudaError_t launch_force3d_iso(const Geom& g, const Phys<R>& p, const StepIO<R>&
 {
     // (param >> 16) & 15: 0 = one lane on 28x12 tiles (FP32: two CTAs per SM),
     // 1 = one lane on 28x28 tiles, 3 = one lane on 28x12 tiles at one CTA per
-    // SM, 4 = two z-lanes in packed FP32x2 on 28x12 tiles (1, 3, 4: FP32 only).
+    // SM, 4 = two z-lanes in packed FP32x2 on 28x12 tiles (1, 3, 4: FP32 only);
+    // 2 = as 0, at automatic heights too.
     // With no planes per segment given either, FP32 takes the packed form: it
     // is the fastest from 64^3 up (64^3: 18.9 us against 29.7 for one lane with
     // segments of 16 planes, 128^3 63 / 66, 250 x 243 x 190 241 / 284, 384^3

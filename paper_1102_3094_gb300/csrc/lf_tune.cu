@@ -73,7 +73,8 @@ std::vector<std::pair<int, int>> candidates(const lf_ctx* c)
     for (int zc : phis) {
         if (zc > g.nz) continue;
         if (iso) {                                   // sliding-sum force pass: two packed z-lanes, one lane on 28x12 (two or one CTA per SM) or 28x28
-            const int sels32[] = {4, 0, 1, 3}, sels64[] = {0};
+            // (2, not 0: one lane at automatic heights too, where 0 means the packed form)
+            const int sels32[] = {4, 2, 1, 3}, sels64[] = {0};
             const int* sels = c->prec == LF_FP32 ? sels32 : sels64;
             const int nsel = c->prec == LF_FP32 ? 4 : 1;
             const int lanes[] = {0, 48, 64, 96, 128, 192};   // planes per lane of the packed form
