@@ -345,19 +345,6 @@ __device__ __forceinline__ void tsub2d_site(const Geom& g, const Phys<R>& p, con
     Tout[site] = t0 + p.dxi * (Tin[y * pitch + xl] + Tin[y * pitch + xr] + tu + td - R(4) * t0);
 }
 
-// Segment height for a lattice: about four CTAs of four warps per SM
-// (param > 0 overrides).
-inline int march_rows_for(int nx, int ny, int U, int param)
-{
-    if (param > 0) return param < ny ? param : ny;
-    const int strips = (nx + U - 1) / U;
-    const int target = 152 * 4;
-    int h = (int)(((int64_t)ny * strips + target - 1) / target);
-    if (h < 12) h = 12;
-    if (h > ny) h = ny;
-    return h;
-}
-
 // Rows per lane for the one-lane marches.  Co-resident CTAs share an SM's
 // issue rate, so the step takes about (CTAs per SM, rounded up) x (rows per
 // lane + 4 pipeline iterations); the smallest such cost wins among heights
