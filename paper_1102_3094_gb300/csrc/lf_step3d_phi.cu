@@ -11,7 +11,7 @@
 // by one shuffle each way (a scalar load where a row of lanes ends),
 // z-neighbours from registers; the two stencils read 13 and 17 vectors per
 // plane.  No shared memory, no barriers.  At the register counts this takes
-// (79 and 138) too few loads are in flight to cover DRAM latency, so each
+// (122 and 153) too few loads are in flight to cover DRAM latency, so each
 // plane is asked for in L2 one iteration before it is loaded: 308 -> 273 us
 // (compact, 98 % of the measured copy bandwidth) and 426 -> 373 us (isotropic,
 // 72 %; the rest is its 440 instructions per 128 sites at 12 warps per SM).
