@@ -216,9 +216,20 @@ def run_reference(args):
     return 0
 
 
-def traffic_for(kernel_key: str):
-    """DRAM bytes per launch from the committed ncu summary, if it still
-    describes the current kernel source."""
+def traffic_for(kernel: str, param: int):
+    """(DRAM bytes per launch, the shape they were captured at) from the committed
+    ncu summary, if it still describes the current kernel source: those of the
+    shape of `param` (key suffix _p<param>), else of the default shape (no suffix),
+    which moves the same fields; (None, None) without either."""
+    for shape, key in ((f"param {param}" if param else "default", f"{kernel}_p{param}" if param else kernel),
+                       ("default", kernel)):
+        b = _captured_bytes(key)
+        if b is not None:
+            return b, shape
+    return None, None
+
+
+def _captured_bytes(kernel_key: str):
     import hashlib
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
@@ -766,9 +777,9 @@ def run_ours(args):
         kname = {"march": "k_march2d", "march2": "k_march2d_x2", "tile": "k_step2d"}[variant]
     if kname.startswith("k_march2d") and kname.endswith("x2") and prec == "fp64":
         kname = kname[:-3]                  # the packed kernels are FP32 only
+    traffic, traffic_shape = traffic_for(f"{kname}_{prec}_{nx}", param)
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            # ncu DRAM bytes per kernel shape (key suffix _p<param>; no suffix: the default shape)
-            "traffic": traffic_for(f"{kname}_{prec}_{nx}" + (f"_p{param}" if param else "")), "peak_kind": peak_kind,
+            "traffic": traffic, "traffic_shape": traffic_shape, "peak_kind": peak_kind,
             "algorithmic_bytes_per_site": bps,
             "kernel": kname + (f" ({passes} passes; bytes and time of the whole step)" if passes > 1
                                else " (fused phi-chain + LB + FD)"),
@@ -886,10 +897,11 @@ def run_ours(args):
         ts = [a.elapsed_time(b) for a, b in zip(starts, ends)]
         tot = max_over_ranks(sum(ts) / 1e3, dev)
         ach = bps * N * args.steps / tot / 1e9
+        traffic, traffic_shape = traffic_for(f"k_force3d+k_lb3d+k_phi3d_iso_{prec}_{nx}", p_) if v_ == 3 else (None, None)
         stable = {"what": "tau = 3, isotropic 19-point stencils (runs the 20k steps finite); no restores",
                   "value": job_rate(N, args.steps, world, tot), "unit": "MLUPS",
                   "ms_per_step": 1e3 * tot / args.steps, "frac": ach / peak, "achieved_gbs": ach,
-                  "traffic": traffic_for(f"k_force3d+k_lb3d+k_phi3d_iso_{prec}_{nx}_p{p_}") if v_ == 3 else None,
+                  "traffic": traffic, "traffic_shape": traffic_shape,
                   "per_pass": pass_breakdown(sim, True, p_, None) if v_ == 3 else None,
                   "kernel_shape": {"variant": names[v_], "param": p_}, "diag_after": {"rc": sim.diag()["rc"]}}
     if rank == 0:
