@@ -412,25 +412,24 @@ int build(lf_ens* e)
 // Rows per lane of every run before any tuning, one height for all runs of a
 // stencil, with 64-thread CTAs (the better width at 4 to 96 runs of 128^2 to
 // 512^2, both stencils).  Six CTAs fit an SM; CTA b takes the items b, b + B,
-// ... of the list sorted by length, so the step takes what CTA 0 does: per item of
-// l rows about s l + c us, by the warps per scheduler that the round leaves (a
-// last round of few items runs faster).  s and c are those that choose best over
-// 19 batches from 2000 runs of 32^2 to three of 4096^2 at heights of 1 to 512: from
-// the best uniform height 0.3 % on average (compact; 2 % at worst), 0.7 %
-// (isotropic; 3 %), without hydrodynamics 0.3 and 0.2 %.  Against 16 rows: 10 runs
-// of 128^2 to 512^2 45.6 -> 41.3 us a step, 96 runs 313 -> 273, isotropic 411 -> 354.
+// ... of the list sorted by length, so the step takes what CTA 0 does: s l + c us
+// per item of l rows, by the warps per scheduler that the CTAs bring.  s and c
+// are those that choose best over 43 batches -- 4 to 96 runs of 128^2 to 512^2, 2000
+// runs of 32^2 to three of 4096^2 -- at heights of 1 to 512: from the best uniform
+// height 0.3 % on average (compact; 2 % at worst) and 0.4 % (isotropic; 4 %),
+// without hydrodynamics 0.3 and 0.4 % (19 batches).  Against 16 rows: 10 runs of
+// 128^2 to 512^2 45.6 -> 41.3 us a step, 96 runs 313 -> 273, isotropic 411 -> 354.
 void default_rows(lf_ens* e)
 {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     sms = std::max(1, sms);
-    // [hydrodynamics][isotropic][warps per scheduler]; isotropic, one round at two warps: 1.93 and 6
+    // [hydrodynamics][isotropic][warps per scheduler]
     const float row[2][2][4] = {{{0, 0.43f, 0.57f, 0.59f}, {0, 0.44f, 0.52f, 0.63f}},
-                                {{0, 1.16f, 1.30f, 1.57f}, {0, 1.37f, 2.57f, 2.48f}}};
+                                {{0, 1.21f, 1.09f, 1.35f}, {0, 1.83f, 1.90f, 2.08f}}};
     const float lag[2][2][4] = {{{0, 4.96f, 2.46f, 3.13f}, {0, 5.05f, 7.2f, 5.3f}},
-                                {{0, 11.05f, 6.59f, 7.84f}, {0, 5.08f, 26.1f, 6.1f}}};
-    auto warps = [sms](int64_t ctas) { return (int)std::min<int64_t>(3, ((ctas + sms - 1) / sms + 1) / 2); };
+                                {{0, 11.6f, 6.7f, 9.4f}, {0, 23.5f, 8.6f, 12.3f}}};
     for (int iso = 0; iso < 2; ++iso) {
         std::vector<int> members;
         std::map<std::pair<int, int>, int> sizes;                        // (nx, ny): runs
@@ -458,16 +457,13 @@ void default_rows(lf_ens* e)
             }
             std::sort(lanes.begin(), lanes.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
             const int64_t B = std::min<int64_t>(items, 6 * (int64_t)sms);
-            const int full = warps(B), last = warps((items - 1) % B + 1);
-            const bool alone = flow && iso && items == B && full == 2;
+            const int k = (int)std::min<int64_t>(3, ((B + sms - 1) / sms + 1) / 2);
+            const float s1 = row[flow][iso][k], s0 = lag[flow][iso][k];
             float us = 0.f;
             int64_t next = 0, end = 0;                                   // CTA 0's next item; items seen
             for (const auto& l : lanes) {
                 end += l.second;
-                for (; next < end; next += B) {
-                    const int k = next + B < items ? full : last;
-                    us += alone ? 1.93f * l.first + 6.f : row[flow][iso][k] * l.first + lag[flow][iso][k];
-                }
+                for (; next < end; next += B) us += s1 * l.first + s0;
             }
             if (best_us < 0.f || us < best_us) {
                 best_us = us;
