@@ -48,16 +48,14 @@ __device__ __forceinline__ void cp_async_s(void* dst, const void* src)
 // places runs at 0.6 of a full one (an SM's issue rate is then shared by half
 // the CTAs).  The number of segments with the least of that wins; few planes
 // per segment on small lattices, where everything fits in one round and only
-// the length of the march counts.  Over ten lattices from 32 x 32 x 256 to
-// 384^3 and both stencils the packed force pass comes within 4 % (48 x 380 x
-// 90: 13 %) of its best height; segments of at least 16 planes, the rule
-// before, cost 64^3 29.5 us instead of 15.0 (compact) and 32 x 32 x 256 29.2
-// instead of 18.2.  In FP64 the planes before a segment's first cost less (their
-// later stages are skipped, and the FP64 pipe is what counts), so `lag` is 3
-// there with either stencil: over 18 lattices from 24^3 to 256^3, with and
-// without hydrodynamics, 0.2 % over the best height on average and 5 % at worst
-// (compact 96^3).  With the FP32 lags, 256 x 128 x 64 isotropic took one segment
-// of 64 planes, 1.17 times the pass with four of 16.
+// the length of the march counts.  The planes before a segment's first skip their
+// later stages, so `lag` is less than their number: 3 for the one-lane forms.
+// Pass times against the best of all heights, on average and at worst: FP64 0.2 %
+// and 5 % (18 lattices from 24^3 to 256^3, both stencils, with and without
+// hydrodynamics), FP32 on one lane 0.1 to 0.8 % and 5 % (11 lattices from 24^3 to
+// 384^3), packed 2.5 % and 9 % (compact, lag 6), 0.8 % and 4 % (isotropic, lag 8).
+// Segments of at least 16 planes, the rule before, cost 64^3 29.5 us instead of
+// 15.0 (compact) and 32 x 32 x 256 29.2 instead of 18.2.
 inline int march3_planes(int64_t tiles, int nz, int lanes, int lag, int res, int sms)
 {
     int best = nz;

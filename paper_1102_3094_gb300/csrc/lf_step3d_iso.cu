@@ -744,7 +744,7 @@ cudaError_t launch_force_iso(const Geom& g, const Phys<R>& p, const StepIO<R>& i
     if (Hz <= 0) {
         int sms = 0;
         if ((e = device_sms(&sms)) != cudaSuccess) return e;
-        Hz = march3_planes(tiles, g.nz, 1, sizeof(R) == 4 ? 8 : 3, MINB, sms);
+        Hz = march3_planes(tiles, g.nz, 1, 3, MINB, sms);
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);

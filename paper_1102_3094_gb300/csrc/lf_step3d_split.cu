@@ -587,7 +587,7 @@ cudaError_t launch_force(const Geom& g, const Phys<R>& p, const StepIO<R>& io, c
     if (Hz <= 0) {
         int sms = 0;
         if ((e = device_sms(&sms)) != cudaSuccess) return e;
-        Hz = sizeof(R) == 4 ? march3_planes(tiles, g.nz, 1, 5, 2, sms) : march3_planes(tiles, g.nz, 1, 3, 1, sms);
+        Hz = march3_planes(tiles, g.nz, 1, 3, sizeof(R) == 4 ? 2 : 1, sms);
     }
     if (Hz > g.nz) Hz = g.nz;
     dim3 grid((g.nx + TX - 1) / TX, (g.ny + TY - 1) / TY, (g.nz + Hz - 1) / Hz);
