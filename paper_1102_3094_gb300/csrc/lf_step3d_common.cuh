@@ -52,8 +52,8 @@ __device__ __forceinline__ void cp_async_s(void* dst, const void* src)
 // later stages, so `lag` is less than their number: 3 for the one-lane forms.
 // Pass times against the best of all heights, on average and at worst: FP64 0.2 %
 // and 5 % (18 lattices from 24^3 to 256^3, both stencils, with and without
-// hydrodynamics), FP32 on one lane 0.1 to 0.8 % and 5 % (11 lattices from 24^3 to
-// 384^3), packed 2.5 % and 9 % (compact, lag 6), 0.8 % and 4 % (isotropic, lag 8).
+// hydrodynamics), FP32 on one lane 1 to 4 % and 14 % (11 lattices from 24^3 to
+// 384^3), packed 5 % and 15 % (compact, lag 6), 2 % and 6 % (isotropic, lag 8).
 // Segments of at least 16 planes, the rule before, cost 64^3 29.5 us instead of
 // 15.0 (compact) and 32 x 32 x 256 29.2 instead of 18.2.
 inline int march3_planes(int64_t tiles, int nz, int lanes, int lag, int res, int sms)
