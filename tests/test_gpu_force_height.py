@@ -23,7 +23,7 @@ def test_automatic_height(precision, stencil, form, dims):
     for h in (0, 3, 9, 11, 16, 22, 29, 32):
         sim.set_variant("split3", form << 16 | h)
         ms[h] = float("inf")
-        for _ in range(8):
+        for _ in range(30):
             sim.step(1)
             ms[h] = min(ms[h], sim.pass_times()[0])
     sim.close()
